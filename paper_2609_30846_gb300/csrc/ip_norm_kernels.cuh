@@ -85,7 +85,7 @@ __device__ __forceinline__ uint32_t recip_2pow31(unsigned long long s64) {
     const long long s = static_cast<long long>(s64);
     const int L = 64 - __clzll(s);
     const long long x = s << (22 - L);
-    long long r = (51539607552ll - 8192ll * x) / 17;   // 2^30 (48 - 32 X) / 17
+    long long r = 3031741620ll - ((x * 123362) >> 8);   // 2^30 (48 - 32 X) / 17
 #pragma unroll
     for (int it = 0; it < 3; ++it) {
         const long long e = (1ll << 52) - x * r;       // |e| < 2^48
