@@ -3,25 +3,34 @@
 // output channel.  Integer arithmetic only: no floating-point type and no
 // division by a run-time value.
 //
-// Persistent kernel: one CTA per SM takes the 128 x 128 tiles of Y (128
-// frames x 128 output channels) round-robin.  With a row-major X the frames
-// of all utterances form one axis of B T rows; with a head-split X a tile
-// stays inside one utterance.  A producer warp streams K in stages of 128
-// bytes: the 128 x 128 int8 tiles of X and W land through TMA with the
-// 128-byte swizzle in a ring of four stages that runs on across tiles, so
-// the next tile's first stages load during the current tile's epilogue.
-// The integer MMA pipe and the dp4a pipe of an SM sub-partition work at the
-// same time, so a tile's channels are split between them: eight MMA warps
-// (2 along the frames x 4 along the channels, 64 x 16 each) take channels
-// 0-63 with the integer warp MMA (mma.sync m16n8k32 s8 x s8 -> s32, from
-// ldmatrix; sm_103a has no integer tcgen05 kind), and eight dp4a warps
-// (16 frames each) take channels 64-127 with dp4a on the same stages.  The
-// epilogue adds the int32 bias, multiplies by m[n] in int64, shifts right by
-// 31 + s[n] with rounding, clamps to [-127, 127] (and, in the feed-forward
-// variant, applies the minimax integer Swish); the MMA warps write their
-// 64 x 16 bytes through shared memory as 16-byte row segments, the dp4a
-// warps their 8-byte row segments directly, either row-major [B][T][N] or
-// head-split [G][B][N/G/128][T][128].
+// What bounds it: the integer MMA pipe (mma.sync m16n8k32 s8, about 65 cycles
+// each on an SM sub-partition) and the dp4a pipe (two cycles a warp), which
+// work at the same time and reach 157 and 159 TOPS alone, 289 together.  So
+// a CTA is four MMA warps and four dp4a warps, one of each on every
+// sub-partition, and two CTAs share an SM (128 registers a thread), so that
+// one computes while the other starts or finishes a tile.
+//
+// One CTA computes one tile of Y, in one of four shapes that the host picks by
+// the size of the problem (64 x 128 down to 32 x 32 frames x channels).  The K
+// axis streams in stages of 128 bytes: TMA lands the X rows and W rows of a
+// stage with the 128-byte swizzle.  The warps form groups that each cover the
+// whole tile, and a group takes one stage of K at a time on its pipe (as many
+// groups as the tile is small: a 32 x 32 tile runs eight, so that even one
+// tile per SM keeps both pipes of all sub-partitions busy).  The groups'
+// partial sums meet in shared memory, where all eight warps requantise them:
+// add the int32 bias, multiply by m[n] in int64, shift right by 31 + s[n] with
+// rounding, clamp to [-127, 127], and apply the minimax integer Swish, the
+// gated unit or the residual addition; four channels per lane, row-major
+// [B][T][N] or head-split [G][B][N/G/128][T][128].  With a row-major X the
+// frames of all utterances form one axis of B T rows; with a head-split X a
+// tile stays inside one utterance.
+//
+// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 9.1 us, 12000 frames
+// 460 -> 451 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 9.3 us,
+// 1332 frames 87.9 -> 57.8 us, 12000 frames 431 -> 410 us (before: one
+// persistent CTA of 17 warps per SM over 128 x 128 tiles, the channels of a
+// tile split between the pipes: a short batch filled 8 to 32 of the SMs, and
+// every lane computed the address of each of its shared loads).
 #pragma once
 
 #include <cuda.h>
@@ -33,35 +42,49 @@ namespace ipl {
 
 using namespace ipk;
 
-constexpr int BM = 128;                 // frames per CTA
-constexpr int BN = 128;                 // output channels per CTA
+constexpr int THREADS = 256;            // four MMA warps and four dp4a warps
 constexpr int BK = 128;                 // K bytes per stage
-constexpr int NCW = 8;                  // MMA warps: 2 (frames) x 4 (channels)
-constexpr int NDW_LOG2 = 3;
-constexpr int NDW = 1 << NDW_LOG2;      // dp4a warps, along the frames (two per SM sub-partition)
-constexpr int DW_ROWS = BM >> NDW_LOG2; // frames of one dp4a warp
-constexpr int RI = DW_ROWS >> 2;        // frames of one dp4a lane (four row groups of lanes)
-constexpr int MMA_COLS = 64;            // channels 0 .. 63 of a tile on the MMA pipe, the rest on dp4a
-constexpr int DW_UNROLL = 2;     // k chunks of a stage unrolled in the dp4a loop
-constexpr int THREADS = (NCW + NDW + 1) * 32;
-constexpr int STAGES = 4;
-constexpr int A_BYTES = BM * BK;
-constexpr int B_BYTES = BN * BK;
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int OUT_ROW = 48;             // staged output row of an MMA warp: 16 bytes, stride 48 (3 x 16: rows spread over the bank groups)
-constexpr int OUT_WARP_BYTES = 64 * OUT_ROW;
-constexpr int SMEM_OUT = STAGES * STAGE_BYTES;
-constexpr int SMEM_BARS = SMEM_OUT + NCW * OUT_WARP_BYTES;
-constexpr int SMEM_LUT = SMEM_BARS + 8 * (2 * STAGES);     // Swish of every int8 z
-constexpr int SMEM_BYTES = SMEM_LUT + 256;
-constexpr int SMEM_LAUNCH = SMEM_BYTES + 1024;   // + alignment of the dynamic base
+constexpr int MAX_SLOTS = 24;           // stages of the largest ring
+
+__host__ __device__ constexpr int lg2(int x) { return x <= 1 ? 0 : 1 + lg2(x >> 1); }
+
+// Shape of one CTA's work.  A unit is what one warp accumulates: 2048
+// outputs (64 x 32 or 32 x 64; 64 per lane) or, for the smallest tile, 1024.
+// The warps whose units cover the tile once form a group; the groups take
+// the K stages in turn, so a group's accumulators are partial sums over its
+// stages, added through shared memory at the end.
+template <int TM_, int TN_>
+struct Shape {
+    static constexpr int TM = TM_, TN = TN_;      // frames x channels
+    static constexpr int OUT = TM * TN;
+    static constexpr int UNIT = OUT >= 2048 ? 2048 : 1024;
+    static constexpr int WPG = OUT >> lg2(UNIT);  // warps per group
+    static constexpr int NG = 8 >> lg2(WPG);      // groups, half of them on each pipe
+    static constexpr int MU_M = UNIT == 1024 ? 32 : (TM >= 64 ? 64 : 32);   // MMA unit
+    static constexpr int MU_N = UNIT >> lg2(MU_M);
+    static constexpr int DU_M = 32;                                         // dp4a unit
+    static constexpr int DU_N = UNIT >> lg2(DU_M);
+    static constexpr int A_BYTES = TM * BK;
+    static constexpr int STAGE = (TM + TN) * BK;
+    static constexpr int LPR = TN >> 2;           // epilogue: lanes per row (four channels each)
+    static constexpr int RPW = 32 >> lg2(LPR);    // rows a warp finishes at a time
+    static constexpr int ROUNDS = TM >> lg2(8 * RPW);
+    static constexpr int CONSTS = 0;              // bias, multiplier, shift of the TN channels
+    static constexpr int LUT = CONSTS + 3 * 4 * TN;
+    static constexpr int BARS = LUT + 256;
+    static constexpr int SLOT_INFO = BARS + 8 * MAX_SLOTS;   // per slot: uses issued, end mark, warps done
+    static constexpr int NEXT = SLOT_INFO + 12 * MAX_SLOTS;    // next stage to claim
+    static constexpr int RING = (NEXT + 4 + 1023) & ~1023;
+    // shared memory of a CTA with pg stages per group (+ alignment of the base)
+    static constexpr int smem(int pg) { return RING + pg * NG * STAGE + 1024; }
+    static_assert(WPG <= 4 && NG >= 2, "groups");
+    static_assert((STAGE & 1023) == 0 && (A_BYTES & 1023) == 0, "128-byte swizzle");
+};
 
 constexpr int LAYOUT_ROWS = 0;
 constexpr int LAYOUT_HEADS = 1;
 constexpr int ERR_PARAM = 16;           // a multiplier, shift or bias out of its domain
 
-static_assert(STAGE_BYTES % 1024 == 0, "128-byte swizzle needs 1024-byte aligned tiles");
-static_assert((STAGES & (STAGES - 1)) == 0, "stage index by mask");
 
 struct LinearParams {
     const int32_t *bias;      // [N] or nullptr
@@ -69,39 +92,40 @@ struct LinearParams {
     const int32_t *s;         // [N]
     int8_t *y;
     int B, T, K, N;
-    int ntn;                  // N / 128 channel tiles
+    int ntn;                  // channel tiles
     int tpu;                  // frame tiles per utterance (head-split X)
-    unsigned ntiles;          // all tiles
     unsigned long long magic_ntn, magic_T, magic_tpu;   // exact division constants
     int heads_per_group;      // N / G / 128 (head-split output)
     int y_layout;
     int x_layout;
+    int epi;                  // EPI_*
+    int pg;                   // ring stages per group
     int *err;
     long long timeout_cycles;
-    // minimax Swish of the requantised output (Eqs. 12-13), SWISH kernels only
+    // minimax Swish of the requantised output (Eqs. 12-13), EPI_SWISH / EPI_GLU
     int sw_qc, sw_qone, sw_m, sw_e;
-    // residual addition of the output to res (Eqs. 1-4), RES kernels only
+    // residual addition of the output to res (Eqs. 1-4), EPI_RES
     const int8_t *res;        // [B][T][N], row-major like the output
     int res_mx, res_my, res_s;
 };
 
 struct Tile {
-    int nt;        // channel tile
-    int b, t0;     // utterance and frame of the first row
+    int n0;        // first channel
+    int b, t0;     // utterance and frame of the first row (head-split X)
     int m0;        // flat row of the first row (b T + t0)
 };
 
+template <class C>
 __device__ __forceinline__ Tile tile_of(unsigned idx, const LinearParams &p) {
     Tile L;
     const unsigned mt = udiv_magic(idx, p.magic_ntn);
-    L.nt = static_cast<int>(idx - mt * static_cast<unsigned>(p.ntn));
+    L.n0 = static_cast<int>(idx - mt * static_cast<unsigned>(p.ntn)) * C::TN;
     if (p.x_layout == LAYOUT_ROWS) {
-        L.m0 = static_cast<int>(mt) * BM;
-        L.b = static_cast<int>(udiv_magic(static_cast<unsigned>(L.m0), p.magic_T));
-        L.t0 = L.m0 - L.b * p.T;
+        L.m0 = static_cast<int>(mt) * C::TM;
+        L.b = L.t0 = 0;
     } else {
         L.b = static_cast<int>(udiv_magic(mt, p.magic_tpu));
-        L.t0 = (static_cast<int>(mt) - L.b * p.tpu) * BM;
+        L.t0 = (static_cast<int>(mt) - L.b * p.tpu) * C::TM;
         L.m0 = L.b * p.T + L.t0;
     }
     return L;
@@ -137,56 +161,105 @@ constexpr int EPI_SWISH = 1;   // + minimax Swish
 constexpr int EPI_GLU = 2;     // interleaved pairs (a_c, b_c) -> a_c sigma(b_c)
 constexpr int EPI_RES = 3;     // requantised int8, then the residual addition to res
 
-// Offset in Y of tile row r (0 .. BM - 1) at tile column col, or -1 past the
-// last frame.  Row-major Y [B][T][N] (or [B][T][N / 2] for the gated unit,
-// with `width` its row length) or head-split Y [G][B][N / G / 128][T][128];
-// hh, grp: the tile's head within its group and the group.
-__device__ __forceinline__ long long y_offset(const LinearParams &p, const Tile &L, int r, int col,
-                                              int width, int hh, int grp) {
-    int b = L.b, t = L.t0 + r;
-    if (p.x_layout == LAYOUT_ROWS) {
-        if (L.m0 + r >= p.B * p.T) return -1;
-        if (p.y_layout == LAYOUT_ROWS)
-            return static_cast<long long>(L.m0 + r) * width + col;
-        while (t >= p.T) {   // rows of a flat tile may run into later utterances
-            t -= p.T;
-            ++b;
+// Eq. 7 for one accumulator (with its bias): max(round(m acc / 2^(31 + s)), -127)
+// with rnd = 2^(30 + s); the callers clamp at 127 (a saturating pack).
+// |m acc| < 2^62, so the quotient by 2^31 is a 32-bit value (funnel
+// shift) and the rest is a shift by s.
+__device__ __forceinline__ int requant(int acc, int cm, int cs, long long rnd) {
+    const long long v = static_cast<long long>(cm) * acc + rnd;
+    const int h = static_cast<int>(__funnelshift_r(static_cast<uint32_t>(v),
+                                                   static_cast<uint32_t>(v >> 32), 31));
+    return max(h >> cs, -127);
+}
+
+// One stage of a dp4a unit: lane (rg, cg) of RG row and CG channel groups
+// (RG CG = 32) accumulates the rows rg + RG i and the channels cg + CG j.  All
+// lanes take the same 16-byte k chunk at a time: chunk c of row r sits at
+// 128 r + 16 (c ^ (r & 7)), so the lanes of a quarter-warp load phase read
+// either one address or distinct bank groups, and since r & 7 takes one value
+// per lane (two where RG or CG is 4) the sixteen loads of a chunk need three
+// addresses and immediate offsets.  (With lanes on consecutive rows and
+// channels every load had an address of its own to compute: 128 TOPS for the
+// loop alone against 143 now, 243 against 263 beside the MMA warps.)  The
+// loads run ahead: the next W chunk during the current one's products, the
+// next X chunks behind the last use of the current ones.
+template <int RI, int CG>
+__device__ __forceinline__ void dp4a_stage(int (&acc)[RI][8], uint32_t at, uint32_t bt, int rg,
+                                           int cg) {
+    constexpr int RG = 32 >> lg2(CG);
+    uint32_t a0 = (at + rg * 128) | (static_cast<uint32_t>(rg) << 4), a1 = a0 ^ (RG == 4 ? 64u : 0u);
+    uint32_t b0 = (bt + cg * 128) | (static_cast<uint32_t>(cg) << 4), b1 = b0 ^ (CG == 4 ? 64u : 0u);
+    uint4 a[RI], b;
+#pragma unroll
+    for (int i = 0; i < RI; ++i) a[i] = lds128(((i & 1) ? a1 : a0) + i * (RG * 128));
+    b = lds128(b0);
+#pragma unroll 1
+    for (uint32_t c = 0; c < 128; c += 16) {
+        const uint32_t d = c ^ ((c + 16) & 127);   // to the next chunk (the first again after the last)
+        const uint32_t a0n = a0 ^ d, a1n = a1 ^ d, b0n = b0 ^ d;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint4 bn = j < 7 ? lds128(((j & 1) ? b0 : b1) + (j + 1) * (CG * 128)) : lds128(b0n);
+#pragma unroll
+            for (int i = 0; i < RI; ++i) {
+                acc[i][j] = __dp4a(static_cast<int>(a[i].x), static_cast<int>(b.x), acc[i][j]);
+                acc[i][j] = __dp4a(static_cast<int>(a[i].y), static_cast<int>(b.y), acc[i][j]);
+                acc[i][j] = __dp4a(static_cast<int>(a[i].z), static_cast<int>(b.z), acc[i][j]);
+                acc[i][j] = __dp4a(static_cast<int>(a[i].w), static_cast<int>(b.w), acc[i][j]);
+                if (j == 7) a[i] = lds128(((i & 1) ? a1n : a0n) + i * (RG * 128));
+            }
+            b = bn;
         }
-    } else if (t >= p.T) {
-        return -1;
+        a0 = a0n;
+        a1 = a1n;
+        b0 = b0n;
+        b1 ^= d;
     }
-    if (p.y_layout == LAYOUT_ROWS) return (static_cast<long long>(b) * p.T + t) * width + col;
-    return (((static_cast<long long>(grp) * p.B + b) * p.heads_per_group + hh) * p.T + t) * 128 + col;
 }
 
-// Per-channel constants of Eq. 7 for channel n, clipped into their domain
-// (bad is set when one was out of it).
-__device__ __forceinline__ void channel_consts(const LinearParams &p, int n, int &cb, int &cm,
-                                               int &ce, bool &bad) {
-    int bi = p.bias != nullptr ? __ldg(p.bias + n) : 0;
-    int mi = __ldg(p.m + n);
-    int si = __ldg(p.s + n);
-    if (mi < 0 || si < 0 || si > 31 || bi >= (1 << 30) || bi <= -(1 << 30)) {
-        bad = true;
-        mi = mi < 0 ? 0 : mi;
-        si = si < 0 ? 0 : (si > 31 ? 31 : si);
-        bi = 0;
+// One stage of an MMA unit of MI m16 x NI n8 tiles.
+template <int MI, int NI>
+__device__ __forceinline__ void mma_stage(int (&acc)[MI][NI][4], uint32_t at, uint32_t bt, int lane) {
+    const int lm_row = lane & 7, lm_mat = lane >> 3;
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        uint32_t af[MI][4], bf[NI][2];
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+            ldsm_x4(at + swz(16 * i + (lm_mat & 1) * 8 + lm_row, 2 * ks + (lm_mat >> 1)), af[i][0],
+                    af[i][1], af[i][2], af[i][3]);
+#pragma unroll
+        for (int j = 0; j < NI; j += 2)
+            ldsm_x4(bt + swz(8 * j + (lm_mat >> 1) * 8 + lm_row, 2 * ks + (lm_mat & 1)), bf[j][0],
+                    bf[j][1], bf[j + 1][0], bf[j + 1][1]);
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < NI; ++j) mma_s8s8(acc[i][j], af[i], bf[j][0], bf[j][1]);
     }
-    cb = bi;
-    cm = mi;
-    ce = 31 + si;
 }
 
-// Eq. 7 for one accumulator: clamp(round(m (acc + bias) / 2^(31 + s))).
-__device__ __forceinline__ int requant(int acc, int cb, int cm, int ce) {
-    const long long v = static_cast<long long>(cm) * (acc + cb) + (1ll << (ce - 1));
-    return clamp127(v >> ce);
+// Wrapping increment of a shared-memory counter (0 .. limit), ordered with
+// the accesses before and after it; returns the old value.
+__device__ __forceinline__ uint32_t atom_inc(uint32_t addr, uint32_t limit) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.cta.shared.inc.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(limit) : "memory");
+    return old;
 }
 
-template <int EPI>
-__global__ void __launch_bounds__(THREADS, 1)
+// Word of tile element (row, col) in a group's partial sums: the channel
+// index XORed with the row, so that the fragment stores of an MMA warp (four
+// rows per phase) fall on distinct banks.
+template <int TN>
+__device__ __forceinline__ uint32_t part_at(int row, int col) {
+    return static_cast<uint32_t>(row * TN + (col ^ ((row & 3) << 3))) * 4u;
+}
+
+template <int TM, int TN>
+__global__ void __launch_bounds__(THREADS, 2)
     linear_i8_kernel(const __grid_constant__ CUtensorMap tm_x,
                      const __grid_constant__ CUtensorMap tm_w, const LinearParams prm) {
+    using C = Shape<TM, TN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -194,314 +267,239 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int lane = threadIdx.x & 31;
     const int kt = prm.K / BK;     // BK is a power of two: a shift
 
-    const uint32_t base = smem_u32(smem);
-    const uint32_t bars = base + SMEM_BARS;
-    auto full_bar = [&](int s) { return bars + 8u * s; };
-    auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
-    auto stage = [&](int s) { return base + s * STAGE_BYTES; };
+    const uint32_t base = smem_u32(smem), ring = base + C::RING;
+    auto full_bar = [&](int s) { return base + C::BARS + 8u * s; };
+    volatile int *issued = reinterpret_cast<int *>(smem + C::SLOT_INFO);
+    volatile int *ended = issued + MAX_SLOTS;
+    int *next = reinterpret_cast<int *>(smem + C::NEXT);
+    const uint32_t done = base + C::SLOT_INFO + 8 * MAX_SLOTS;   // per slot: warps done with its stage
+    const uint8_t *swish_lut = smem + C::LUT;
+    const int slots = C::NG * prm.pg;
 
-    const uint32_t lut = base + SMEM_LUT;
-    const uint8_t *swish_lut = smem + SMEM_LUT;
     pdl_launch_dependents();
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full_bar(s), 1);
-            mbar_init(empty_bar(s), NCW + NDW);
-        }
+    if (threadIdx.x < slots) {
+        mbar_init(full_bar(threadIdx.x), 1);
+        sts32(done + 4u * threadIdx.x, 0u);
+        issued[threadIdx.x] = -1;
+        ended[threadIdx.x] = 0;
+        if (threadIdx.x == 0) *next = slots;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (EPI == EPI_SWISH && threadIdx.x < 256) {
-        // the Swish of every int8 input, entry at the byte value of z
-        const int z = static_cast<int>(static_cast<int8_t>(static_cast<uint8_t>(threadIdx.x)));
-        const uint32_t y = static_cast<uint32_t>(swish_i8(z, prm)) & 0xffu;
-        asm volatile("st.shared.u8 [%0], %1;" ::"r"(lut + threadIdx.x), "r"(y) : "memory");
-    }
-    pdl_wait();   // the grid before this one on the stream: complete, memory visible
+    const Tile L = tile_of<C>(blockIdx.x, prm);
     __syncthreads();
+    pdl_wait();   // the grid before this one on the stream: complete, memory visible
 
-    // ---------------------------------------------------------- producer
-    // Use u of the ring: stage u & 3, phase (u / 4) & 1.
-    if (warp == NCW + NDW) {
-        unsigned u = 0, landed_from = 0;
-        bool ok = true;
-        for (unsigned idx = blockIdx.x; idx < prm.ntiles && ok; idx += gridDim.x) {
-            const Tile L = tile_of(idx, prm);
-            for (int it = 0; it < kt; ++it, ++u) {
-                const int s = static_cast<int>(u & (STAGES - 1));
-                if (u >= STAGES &&
-                    !warp_wait(empty_bar(s), ((u / STAGES) - 1) & 1, prm.timeout_cycles)) {
-                    if (lane == 0) atomicOr(prm.err, 2);
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) {
-                    mbar_expect_tx(full_bar(s), STAGE_BYTES);
-                    if (prm.x_layout == LAYOUT_ROWS)
-                        tma_load_2d(stage(s), &tm_x, it * BK, L.m0, full_bar(s));
-                    else
-                        tma_load_4d(stage(s), &tm_x, 0, L.t0, it, L.b, full_bar(s));
-                    tma_load_2d(stage(s) + A_BYTES, &tm_w, it * BK, L.nt * BN, full_bar(s));
-                }
-            }
+    // Warps 0-3 run the integer MMA pipe, 4-7 the dp4a pipe (one of each on
+    // every SM sub-partition).  Each group has pg slots of the ring (group g:
+    // slots g, g + NG, ...) and uses them in turn; when a slot has been
+    // consumed, the group's first warp claims the next stage of K for it, so
+    // the faster pipe takes more stages.  A slot without a stage is marked
+    // ended and its barrier completed without a copy.
+    const bool on_mma = warp < 4;
+    const int gi = C::WPG == 1 ? (warp & 3) : (C::WPG == 2 ? (warp & 3) >> 1 : 0);
+    const int u = (warp & 3) & (C::WPG - 1);
+    const int grp = 2 * gi + (on_mma ? 0 : 1);
+    auto issue = [&](int it, int slot, int use) {
+        if (it >= kt) {
+            ended[slot] = 1;
+            issued[slot] = -1;   // its copies have been consumed
+            mbar_arrive(full_bar(slot));
+            return;
         }
-        if (!ok) {
-            // let the copies in flight land before the CTA exits
-            landed_from = u > STAGES ? u - STAGES : 0;
-            for (unsigned v = landed_from; v < u; ++v)
-                mbar_wait(full_bar(static_cast<int>(v & (STAGES - 1))), (v / STAGES) & 1,
-                          2000000000ll);
+        const uint32_t st = ring + slot * C::STAGE;
+        issued[slot] = use;
+        mbar_expect_tx(full_bar(slot), C::STAGE);
+        if (prm.x_layout == LAYOUT_ROWS)
+            tma_load_2d(st, &tm_x, it * BK, L.m0, full_bar(slot));
+        else
+            tma_load_4d(st, &tm_x, 0, L.t0, it, L.b, full_bar(slot));
+        tma_load_2d(st + C::A_BYTES, &tm_w, it * BK, L.n0, full_bar(slot));
+    };
+    if (u == 0 && lane == 0)
+        for (int slot = grp; slot < slots; slot += C::NG) issue(slot, slot, 0);
+
+    // while the first stages land: the channel constants (clipped into their
+    // domain) and the Swish of every int8 input, entry at the byte value of z
+    int32_t *cst = reinterpret_cast<int32_t *>(smem + C::CONSTS);
+    if (threadIdx.x < TN) {
+        const int n = L.n0 + threadIdx.x;
+        int bi = prm.bias != nullptr ? __ldg(prm.bias + n) : 0;
+        int mi = __ldg(prm.m + n);
+        int si = __ldg(prm.s + n);
+        if (mi < 0 || si < 0 || si > 31 || bi >= (1 << 30) || bi <= -(1 << 30)) {
+            atomicOr(prm.err, ERR_PARAM);
+            mi = mi < 0 ? 0 : mi;
+            si = si < 0 ? 0 : (si > 31 ? 31 : si);
+            bi = 0;
         }
-        return;
+        cst[threadIdx.x] = bi;
+        cst[TN + threadIdx.x] = mi;
+        cst[2 * TN + threadIdx.x] = si;
     }
+    if (prm.epi == EPI_SWISH)
+        smem[C::LUT + threadIdx.x] = static_cast<uint8_t>(
+            swish_i8(static_cast<int>(static_cast<int8_t>(static_cast<uint8_t>(threadIdx.x))), prm));
 
-    const int frames = prm.B * prm.T;
-
-    // ---------------------------------------------------------- dp4a warps
-    // Channels MMA_COLS .. BN - 1 of every tile, rows DW_ROWS dw .. DW_ROWS dw
-    // + DW_ROWS - 1: lane (rg, cg) = (lane / 8, lane % 8) accumulates rows
-    // DW_ROWS dw + RI rg + i (i < RI) and channels MMA_COLS + 8 cg + j (j < 8)
-    // with dp4a on the same stages the MMA warps read.  Each lane walks the
-    // eight 16-byte k chunks of a stage starting at chunk cg: the four lanes
-    // of a channel group then read the same W chunk (one broadcast) and the
-    // eight groups' chunks fall on the eight bank groups of the swizzled
-    // rows, while the X loads of a row group cover every bank group too.
-    if (warp >= NCW) {
-        const int dw = warp - NCW;
-        const int rg = lane >> 3, cg = lane & 7;
-        const int r0 = DW_ROWS * dw + RI * rg;
-        const int r7 = r0 & 7;          // 0 or 4: r7 + i = r7 | i for i < RI
-        const int c0 = MMA_COLS + 8 * cg;
-        unsigned u = 0;
-        for (unsigned idx = blockIdx.x; idx < prm.ntiles; idx += gridDim.x) {
-            const Tile L = tile_of(idx, prm);
-            const int n0 = L.nt * BN;
-            int acc[RI][8];
-#pragma unroll
-            for (int i = 0; i < RI; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = 0;
-            for (int it = 0; it < kt; ++it, ++u) {
-                const int s = static_cast<int>(u & (STAGES - 1));
-                if (!warp_wait(full_bar(s), (u / STAGES) & 1, prm.timeout_cycles)) {
-                    if (lane == 0) atomicOr(prm.err, 1);
-                    return;
-                }
-                const uint32_t abase = stage(s) + r0 * 128;
-                const uint32_t bbase = stage(s) + A_BYTES + c0 * 128;
-#pragma unroll (DW_UNROLL)
-                for (int c = 0; c < 8; ++c) {
-                    const int kc = (c + cg) & 7;
-                    uint4 a[RI];
-#pragma unroll
-                    for (int i = 0; i < RI; ++i)
-                        a[i] = lds128(abase + i * 128 + ((kc ^ (r7 | i)) << 4));
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint4 b = lds128(bbase + j * 128 + ((kc ^ j) << 4));
-#pragma unroll
-                        for (int i = 0; i < RI; ++i) {
-                            acc[i][j] = __dp4a(static_cast<int>(a[i].x), static_cast<int>(b.x), acc[i][j]);
-                            acc[i][j] = __dp4a(static_cast<int>(a[i].y), static_cast<int>(b.y), acc[i][j]);
-                            acc[i][j] = __dp4a(static_cast<int>(a[i].z), static_cast<int>(b.z), acc[i][j]);
-                            acc[i][j] = __dp4a(static_cast<int>(a[i].w), static_cast<int>(b.w), acc[i][j]);
-                        }
-                    }
-                }
-                release_stage(empty_bar(s), lane);
-            }
-
-            // epilogue: eight channels per lane, one 8-byte (4-byte gated)
-            // segment per row, straight to global memory
-            int cb[8], cm[8], ce[8];
-            bool bad = false;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) channel_consts(prm, n0 + c0 + j, cb[j], cm[j], ce[j], bad);
-            if (bad) atomicOr(prm.err, ERR_PARAM);
-            int hh = L.nt, grp = 0;
-            if (prm.y_layout == LAYOUT_HEADS)
-                while (hh >= prm.heads_per_group) {   // at most G - 1 steps
-                    hh -= prm.heads_per_group;
-                    ++grp;
-                }
-#pragma unroll
-            for (int i = 0; i < RI; ++i) {
-                if (EPI == EPI_GLU) {
-                    uint32_t w = 0;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int za = requant(acc[i][2 * q], cb[2 * q], cm[2 * q], ce[2 * q]);
-                        const int zb = requant(acc[i][2 * q + 1], cb[2 * q + 1], cm[2 * q + 1],
-                                               ce[2 * q + 1]);
-                        w |= (static_cast<uint32_t>(glu_i8(za, zb, prm)) & 0xffu) << (8 * q);
-                    }
-                    const long long off = y_offset(prm, L, r0 + i, (n0 + c0) >> 1, prm.N >> 1, hh, grp);
-                    if (off >= 0) *reinterpret_cast<uint32_t *>(prm.y + off) = w;
-                } else {
-                    uint32_t w[2] = {0u, 0u};
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        uint32_t o = static_cast<uint32_t>(requant(acc[i][j], cb[j], cm[j], ce[j])) & 0xffu;
-                        if (EPI == EPI_SWISH) o = swish_lut[o];
-                        w[j >> 2] |= o << (8 * (j & 3));
-                    }
-                    const int col = prm.y_layout == LAYOUT_ROWS ? n0 + c0 : c0;
-                    const long long off = y_offset(prm, L, r0 + i, col, prm.N, hh, grp);
-                    if (off >= 0) {
-                        if (EPI == EPI_RES) {
-                            const uint2 xr = *reinterpret_cast<const uint2 *>(prm.res + off);
-                            w[0] = residual4(xr.x, w[0], prm.res_mx, prm.res_my, prm.res_s);
-                            w[1] = residual4(xr.y, w[1], prm.res_mx, prm.res_my, prm.res_s);
-                        }
-                        *reinterpret_cast<uint2 *>(prm.y + off) = make_uint2(w[0], w[1]);
-                    }
-                }
-            }
-        }
-        return;
-    }
-
-    // ---------------------------------------------------------- MMA warps
-    // Channels 0 .. MMA_COLS - 1: warp (wm, wn) takes rows 64 wm .. 64 wm +
-    // 63 and channels 16 wn .. 16 wn + 15 (two n8 tiles).
-    const int wm = warp & 1;
-    const int wn = warp >> 1;
-    const int g = lane >> 2, t4 = lane & 3;
-    const int lm_row = lane & 7, lm_mat = lane >> 3;
-    const uint32_t ob = base + SMEM_OUT + warp * OUT_WARP_BYTES;
-
-    unsigned u = 0;
-    for (unsigned idx = blockIdx.x; idx < prm.ntiles; idx += gridDim.x) {
-        const Tile L = tile_of(idx, prm);
-        const int n0 = L.nt * BN;
-
-        int acc[4][2][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-                acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0;
-
-        for (int it = 0; it < kt; ++it, ++u) {
-            const int s = static_cast<int>(u & (STAGES - 1));
-            if (!warp_wait(full_bar(s), (u / STAGES) & 1, prm.timeout_cycles)) {
+    bool ok = true;
+    auto run_stages = [&](auto &&compute) {
+        for (int slot = grp, use = 0;;) {
+            if (!warp_wait(full_bar(slot), use & 1, prm.timeout_cycles)) {
                 if (lane == 0) atomicOr(prm.err, 1);
+                ok = false;
                 return;
             }
-            const uint32_t at = stage(s) + (64 * wm) * 128;
-            const uint32_t bt = stage(s) + A_BYTES + (16 * wn) * 128;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                uint32_t af[4][4], bf[2][2];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    ldsm_x4(at + swz(16 * i + (lm_mat & 1) * 8 + lm_row, 2 * ks + (lm_mat >> 1)),
-                            af[i][0], af[i][1], af[i][2], af[i][3]);
-                ldsm_x4(bt + swz((lm_mat >> 1) * 8 + lm_row, 2 * ks + (lm_mat & 1)), bf[0][0],
-                        bf[0][1], bf[1][0], bf[1][1]);
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) mma_s8s8(acc[i][j], af[i], bf[j][0], bf[j][1]);
-            }
-            release_stage(empty_bar(s), lane);
-        }
-
-        // ------------------------------------------------------ epilogue
-        // per-channel constants of this thread's four channels (Eq. 7),
-        // loaded after the main loop so that they hold no registers during it
-        int cb[4], cm[4], ce[4];
-        bool bad = false;
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-                channel_consts(prm, n0 + 16 * wn + 8 * j + 2 * t4 + q, cb[2 * j + q], cm[2 * j + q],
-                               ce[2 * j + q], bad);
-        if (bad) atomicOr(prm.err, ERR_PARAM);
-
-        if (EPI == EPI_GLU) {
-            // pairs (a_c, b_c) in columns (2t, 2t + 1) of each n8 tile: output
-            // channel 4j + t of this warp's 8 (row of 8 bytes)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int rr = 0; rr < 2; ++rr) {
-                        const int za = requant(acc[i][j][2 * rr], cb[2 * j], cm[2 * j], ce[2 * j]);
-                        const int zb = requant(acc[i][j][2 * rr + 1], cb[2 * j + 1], cm[2 * j + 1],
-                                               ce[2 * j + 1]);
-                        const uint32_t o = static_cast<uint32_t>(glu_i8(za, zb, prm)) & 0xffu;
-                        const int r = 16 * i + g + 8 * rr;
-                        asm volatile("st.shared.u8 [%0], %1;" ::"r"(ob + r * OUT_ROW + 4 * j + t4),
-                                     "r"(o)
-                                     : "memory");
-                    }
+            if (ended[slot]) return;
+            compute(ring + slot * C::STAGE);
+            // the last warp of the group to finish refills the slot: nobody waits
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            // 64 rows x 8 bytes: lane -> rows lane, lane + 32
-#pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int r = 32 * it + lane;
-                const int2 v2 = lds64(ob + r * OUT_ROW);
-                const uint2 v = make_uint2(static_cast<uint32_t>(v2.x), static_cast<uint32_t>(v2.y));
-                if (L.m0 + 64 * wm + r < frames) {
-                    const size_t off = static_cast<size_t>(L.m0 + 64 * wm + r) * (prm.N >> 1) +
-                                       (n0 >> 1) + 8 * wn;
-                    *reinterpret_cast<uint2 *>(prm.y + off) = v;
-                }
-            }
-            __syncwarp();
-            continue;
-        }
-
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int rr = 0; rr < 2; ++rr) {
-                    uint32_t two = 0;
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const int c = 2 * j + q;
-                        uint32_t o = static_cast<uint32_t>(requant(acc[i][j][2 * rr + q], cb[c], cm[c],
-                                                                   ce[c])) & 0xffu;
-                        if (EPI == EPI_SWISH) o = swish_lut[o];
-                        two |= o << (8 * q);
-                    }
-                    const int r = 16 * i + g + 8 * rr;
-                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(ob + r * OUT_ROW + 8 * j + 2 * t4),
-                                 "h"(static_cast<unsigned short>(two))
-                                 : "memory");
-                }
-        __syncwarp();
-
-        int hh = L.nt, grp = 0;
-        if (prm.y_layout == LAYOUT_HEADS)
-            while (hh >= prm.heads_per_group) {   // at most G - 1 steps
-                hh -= prm.heads_per_group;
-                ++grp;
-            }
-        // 64 rows x 16 bytes: lane -> rows lane, lane + 32
-#pragma unroll
-        for (int it = 0; it < 2; ++it) {
-            const int r = 32 * it + lane;
-            uint4 v = lds128(ob + r * OUT_ROW);
-            const int col = prm.y_layout == LAYOUT_ROWS ? n0 + 16 * wn : 16 * wn;
-            const long long off = y_offset(prm, L, 64 * wm + r, col, prm.N, hh, grp);
-            if (off >= 0) {
-                if (EPI == EPI_RES) {
-                    const uint4 xr = *reinterpret_cast<const uint4 *>(prm.res + off);
-                    v = make_uint4(residual4(xr.x, v.x, prm.res_mx, prm.res_my, prm.res_s),
-                                   residual4(xr.y, v.y, prm.res_mx, prm.res_my, prm.res_s),
-                                   residual4(xr.z, v.z, prm.res_mx, prm.res_my, prm.res_s),
-                                   residual4(xr.w, v.w, prm.res_mx, prm.res_my, prm.res_s));
-                }
-                *reinterpret_cast<uint4 *>(prm.y + off) = v;
+            if (lane == 0 && (C::WPG == 1 || atom_inc(done + 4u * slot, C::WPG - 1) == C::WPG - 1))
+                issue(atomicAdd(next, 1), slot, use + 1);
+            slot += C::NG;
+            if (slot >= slots) {
+                slot = grp;
+                ++use;
             }
         }
-        __syncwarp();
+    };
+
+    // Partial sums of the group, written over the ring once every warp has
+    // read its last stage.
+    auto all_done = [&]() -> bool {
+        if (__syncthreads_or(ok ? 0 : 1) == 0) return true;
+        if (threadIdx.x == 0)   // let the copies in flight land before the CTA exits
+            for (int s = 0; s < slots; ++s)
+                if (issued[s] >= 0) mbar_wait(full_bar(s), issued[s] & 1, 2000000000ll);
+        return false;
+    };
+    const uint32_t part = ring + grp * (C::OUT * 4);
+    if (on_mma) {
+        constexpr int MI = C::MU_M >> 4, NI = C::MU_N >> 3;
+        constexpr int UL = lg2(TM) - lg2(C::MU_M);   // units along the frames: 1 << UL
+        const int r0 = C::MU_M * (u & ((1 << UL) - 1)), c0 = C::MU_N * (u >> UL);
+        int acc[MI][NI][4];
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < NI; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0;
+        run_stages([&](uint32_t st) {
+            mma_stage<MI, NI>(acc, st + r0 * 128, st + C::A_BYTES + c0 * 128, lane);
+        });
+        if (!all_done()) return;
+        const int g = lane >> 2, t4 = lane & 3;
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = 0; j < NI; ++j)
+#pragma unroll
+                for (int rr = 0; rr < 2; ++rr)
+                    sts64(part + part_at<TN>(r0 + 16 * i + g + 8 * rr, c0 + 8 * j + 2 * t4),
+                          acc[i][j][2 * rr], acc[i][j][2 * rr + 1]);
+    } else {
+        constexpr int CG = C::DU_N >> 3, RI = C::DU_M >> lg2(32 >> lg2(CG));
+        constexpr int UL = lg2(TM) - lg2(C::DU_M);
+        const int rg = lane >> lg2(CG), cg = lane & (CG - 1);
+        const int r0 = C::DU_M * (u & ((1 << UL) - 1)), c0 = C::DU_N * (u >> UL);
+        int acc[RI][8];
+#pragma unroll
+        for (int i = 0; i < RI; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = 0;
+        run_stages([&](uint32_t st) {
+            dp4a_stage<RI, CG>(acc, st + r0 * 128, st + C::A_BYTES + c0 * 128, rg, cg);
+        });
+        if (!all_done()) return;
+#pragma unroll
+        for (int i = 0; i < RI; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                sts32(part + part_at<TN>(r0 + rg + (32 >> lg2(CG)) * i, c0 + cg + CG * j),
+                      static_cast<uint32_t>(acc[i][j]));
+    }
+
+    // ------------------------------------------------------------ epilogue
+    // Lane: four consecutive channels, rows rl, rl + 8 RPW, ...; the loads of
+    // the residual operand go out before the partial sums are awaited.
+    const int cl = 4 * (lane & (C::LPR - 1)), rl = C::RPW * warp + (lane >> lg2(C::LPR));
+    const int col = L.n0 + cl, flat0 = L.m0 + rl;
+    const int frames = prm.x_layout == LAYOUT_ROWS ? prm.B * prm.T : (L.b + 1) * prm.T;
+    const bool glu = prm.epi == EPI_GLU;
+    constexpr int STEP = 8 * C::RPW;
+    // Row-major Y [B][T][width] (width N, N / 2 behind the gated unit), or
+    // head-split Y [G][B][N / G / 128][T][128]: frame t of utterance b.
+    const long long width = glu ? prm.N >> 1 : prm.N;
+    long long off = static_cast<long long>(flat0) * width + (glu ? col >> 1 : col);
+    const bool heads = prm.y_layout == LAYOUT_HEADS;
+    int t = 0;
+    if (heads) {
+        int hh = L.n0 >> 7, gg = 0;
+        while (hh >= prm.heads_per_group) {   // at most G - 1 steps
+            hh -= prm.heads_per_group;
+            ++gg;
+        }
+        const int b = static_cast<int>(udiv_magic(static_cast<unsigned>(flat0), prm.magic_T));
+        t = flat0 - b * prm.T;
+        off = ((((static_cast<long long>(gg) * prm.B + b) * prm.heads_per_group + hh) * prm.T + t) << 7) +
+              (col & 127);
+    }
+    uint32_t xr[C::ROUNDS];
+    if (prm.epi == EPI_RES) {
+#pragma unroll
+        for (int q = 0; q < C::ROUNDS; ++q)
+            if (flat0 + STEP * q < frames)
+                xr[q] = *reinterpret_cast<const uint32_t *>(prm.res + off + STEP * q * width);
+    }
+    __syncthreads();
+    int cb[4], cm[4], cs[4];
+    long long rnd[4];
+    {
+        const uint4 vb = lds128(base + C::CONSTS + 4 * cl);
+        const uint4 vm = lds128(base + C::CONSTS + 4 * (TN + cl));
+        const uint4 vs = lds128(base + C::CONSTS + 4 * (2 * TN + cl));
+        cb[0] = static_cast<int>(vb.x), cb[1] = static_cast<int>(vb.y), cb[2] = static_cast<int>(vb.z), cb[3] = static_cast<int>(vb.w);
+        cm[0] = static_cast<int>(vm.x), cm[1] = static_cast<int>(vm.y), cm[2] = static_cast<int>(vm.z), cm[3] = static_cast<int>(vm.w);
+        cs[0] = static_cast<int>(vs.x), cs[1] = static_cast<int>(vs.y), cs[2] = static_cast<int>(vs.z), cs[3] = static_cast<int>(vs.w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) rnd[e] = 1ll << (30 + cs[e]);
+    }
+#pragma unroll
+    for (int q = 0; q < C::ROUNDS; ++q) {
+        if (flat0 + STEP * q >= frames) break;
+        int a[4] = {cb[0], cb[1], cb[2], cb[3]};
+#pragma unroll
+        for (int g = 0; g < C::NG; ++g) {
+            const uint4 v = lds128(ring + g * (C::OUT * 4) + part_at<TN>(rl + STEP * q, cl));
+            a[0] += static_cast<int>(v.x);
+            a[1] += static_cast<int>(v.y);
+            a[2] += static_cast<int>(v.z);
+            a[3] += static_cast<int>(v.w);
+        }
+        int z[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) z[e] = requant(a[e], cm[e], cs[e], rnd[e]);
+        int8_t *dst = prm.y + off;
+        if (glu) {
+            // channels (a_c, b_c) interleaved: two gated outputs
+            const uint32_t w = (static_cast<uint32_t>(glu_i8(min(z[0], 127), min(z[1], 127), prm)) & 0xffu) |
+                               ((static_cast<uint32_t>(glu_i8(min(z[2], 127), min(z[3], 127), prm)) & 0xffu) << 8);
+            *reinterpret_cast<uint16_t *>(dst) = static_cast<uint16_t>(w);
+        } else {
+            uint32_t w = pack_sat4(z[0], z[1], z[2], z[3]);
+            if (prm.epi == EPI_SWISH)
+                w = swish_lut[w & 0xffu] | (swish_lut[(w >> 8) & 0xffu] << 8) |
+                    (swish_lut[(w >> 16) & 0xffu] << 16) | (static_cast<uint32_t>(swish_lut[w >> 24]) << 24);
+            else if (prm.epi == EPI_RES)
+                w = residual4(xr[q], w, prm.res_mx, prm.res_my, prm.res_s);
+            *reinterpret_cast<uint32_t *>(dst) = w;
+        }
+        if (heads) {
+            off += STEP << 7;
+            for (t += STEP; t >= prm.T; t -= prm.T)   // into the next utterance
+                off += static_cast<long long>(prm.heads_per_group - 1) * prm.T << 7;
+        } else {
+            off += STEP * width;
+        }
     }
 }
 

@@ -241,18 +241,6 @@ __device__ __forceinline__ int residual_one(int x, int y, int m_x, int m_y, int 
     return clamp127(h >> s);
 }
 
-// Residual addition of four packed int8 pairs (byte e of x with byte e of y).
-__device__ __forceinline__ uint32_t residual4(uint32_t x, uint32_t y, int m_x, int m_y, int s) {
-    uint32_t w = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int xa = static_cast<int>(static_cast<int8_t>((x >> (8 * e)) & 0xffu));
-        const int yb = static_cast<int>(static_cast<int8_t>((y >> (8 * e)) & 0xffu));
-        w |= (static_cast<uint32_t>(residual_one(xa, yb, m_x, m_y, s)) & 0xffu) << (8 * e);
-    }
-    return w;
-}
-
 // (c << 16) | (sat8(a) << 8) | sat8(b): two int32 values saturated to
 // [-128, 127] and packed below the low half of c (cvt.pack.sat).
 __device__ __forceinline__ uint32_t pack_sat2(int a, int b, uint32_t c) {
@@ -274,6 +262,21 @@ __device__ __forceinline__ int sbyte(uint32_t w, int e) {
     uint32_t r;
     asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(w), "r"(sel));
     return static_cast<int>(r);
+}
+
+// Residual addition of four packed int8 pairs (byte e of x with byte e of y):
+// residual_one's steps with the upper clamp left to the saturating pack.
+__device__ __forceinline__ uint32_t residual4(uint32_t x, uint32_t y, int m_x, int m_y, int s) {
+    int z[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const long long v = static_cast<long long>(m_x) * sbyte(x, e) +
+                            (static_cast<long long>(m_y) * sbyte(y, e) + (1ll << (30 + s)));
+        const int h = static_cast<int>(__funnelshift_r(static_cast<uint32_t>(v),
+                                                       static_cast<uint32_t>(v >> 32), 31));
+        z[e] = max(h >> s, -127);
+    }
+    return pack_sat4(z[0], z[1], z[2], z[3]);
 }
 
 }  // namespace ipk
