@@ -447,6 +447,23 @@ __device__ __forceinline__ void prob_operand(const uint32_t (&pw)[4], uint32_t (
     af[3] = __byte_perm(pw[2], pw[3], 0x7632);
 }
 
+// Eq. 7 for the four outputs d = 16c + 4t .. + 3 of one row (byte e: n-tile 2c
+// + (e & 1), column 2t + (e >> 1)): |m_o acc| < 2^57 (acc < 255 127 T < 2^26), so
+// the quotient by 2^31 is a 32-bit value; the upper clamp is the pack's.
+__device__ __forceinline__ uint32_t out_word(const int (&a)[4], const int (&b)[4], int rr, int m_o, int sh_o) {
+    const long long rnd = 1ll << (sh_o - 1);
+    const int acc[4] = {a[2 * rr], b[2 * rr], a[2 * rr + 1], b[2 * rr + 1]};
+    int z[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const long long x = static_cast<long long>(m_o) * acc[e] + rnd;
+        z[e] = max(static_cast<int>(__funnelshift_r(static_cast<uint32_t>(x), static_cast<uint32_t>(x >> 32), 31)) >>
+                       (sh_o - 31),
+                   -127);
+    }
+    return pack_sat4(z[0], z[1], z[2], z[3]);
+}
+
 // ------------------------------------------------------- split-tile parts --
 // In a split tile the two warps of a row strip take the key halves
 // [32 hk, 32 hk + 32) of every chunk.  Exchange area in each warp's remap
@@ -520,9 +537,8 @@ __device__ __forceinline__ void send_partial(const int (&oacc)[16][4], uint32_t 
 // per row and d chunk: d = 16c + 4t .. 16c + 4t + 3 for c in 4 HK .. 4 HK + 3.
 template <int HK>
 __device__ __forceinline__ void finish_half(int (&oacc)[16][4], uint32_t pxo, int lane, int wrow0,
-                                            int len, const FusedParams &prm, int b, int h,
-                                            long long m_o, long long half_o) {
-    const int T = prm.T, sh_o = prm.sh_o;
+                                            int len, const FusedParams &prm, int b, int h) {
+    const int T = prm.T;
     const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -536,15 +552,8 @@ __device__ __forceinline__ void finish_half(int (&oacc)[16][4], uint32_t pxo, in
         int8_t *dst = prm.out + out_offset(prm, b, h, row) + 4 * t4;
 #pragma unroll
         for (int c = 4 * HK; c < 4 * HK + 4; ++c) {
-            uint32_t w = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                // byte e: d = 16c + 4t + e = n-tile 2c + (e & 1), column 2t + (e >> 1)
-                const long long x = m_o * oacc[2 * c + (e & 1)][2 * rr + (e >> 1)] + half_o;
-                const int o = row < len ? clamp127(x >> sh_o) : 0;
-                w |= (static_cast<uint32_t>(o) & 0xffu) << (8 * e);
-            }
-            *reinterpret_cast<uint32_t *>(dst + 16 * c) = w;
+            *reinterpret_cast<uint32_t *>(dst + 16 * c) =
+                row < len ? out_word(oacc[2 * c], oacc[2 * c + 1], rr, prm.m_o, prm.sh_o) : 0u;
         }
     }
 }
@@ -896,20 +905,12 @@ __device__ __forceinline__ bool consume_whole(const FusedParams &prm, const Item
     // d = 16c + 4t .. 16c + 4t + 3 (n-tiles 2c, 2c + 1, columns 2t, 2t + 1).
     // The d chunks go in the order their last MMAs were issued, so the
     // first ones are requantised while the pipe finishes the others.
-    const long long m_o = prm.m_o;
-    const long long half_o = 1ll << (prm.sh_o - 1);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
             const int row = wrow0 + g + 8 * rr;
-            uint32_t w = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const long long x = m_o * oacc[2 * c + (e & 1)][2 * rr + (e >> 1)] + half_o;
-                const int o = row < len ? clamp127(x >> prm.sh_o) : 0;
-                w |= (static_cast<uint32_t>(o) & 0xffu) << (8 * e);
-            }
+            const uint32_t w = row < len ? out_word(oacc[2 * c], oacc[2 * c + 1], rr, prm.m_o, prm.sh_o) : 0u;
             if (row < T)
                 *reinterpret_cast<uint32_t *>(prm.out + out_offset(prm, it.b, it.h, row) + 4 * t4 +
                                               16 * c) = w;
@@ -1082,12 +1083,10 @@ __device__ __forceinline__ bool consume_half(const FusedParams &prm, const Item 
         if (lane == 0) atomicOr(prm.err, ERR_TIMEOUT_READY);
         return false;
     }
-    const long long m_o = prm.m_o;
-    const long long half_o = 1ll << (prm.sh_o - 1);
     if (hk == 0)
-        finish_half<0>(oacc, xpart + XO_OFF, lane, wrow0, len, prm, it.b, it.h, m_o, half_o);
+        finish_half<0>(oacc, xpart + XO_OFF, lane, wrow0, len, prm, it.b, it.h);
     else
-        finish_half<1>(oacc, xpart + XO_OFF, lane, wrow0, len, prm, it.b, it.h, m_o, half_o);
+        finish_half<1>(oacc, xpart + XO_OFF, lane, wrow0, len, prm, it.b, it.h);
     // both warps are done reading the partner's area before either reuses its own
     __syncwarp();
     if (lane == 0) mbar_arrive(pair);
@@ -1340,8 +1339,6 @@ __device__ __forceinline__ bool consume_quarter(const FusedParams &prm, const It
     }
 
     // Eq. 7 and the stores of d chunks 2w, 2w + 1 (n-tiles 4w .. 4w + 3)
-    const long long m_o = prm.m_o;
-    const long long half_o = 1ll << (prm.sh_o - 1);
     const int T = prm.T;
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
@@ -1350,13 +1347,7 @@ __device__ __forceinline__ bool consume_quarter(const FusedParams &prm, const It
         for (int rr = 0; rr < 2; ++rr) {
             const int row = wrow0 + g + 8 * rr;
             if (row >= T) continue;
-            uint32_t w = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const long long x = m_o * oacc[2 * cc + (e & 1)][2 * rr + (e >> 1)] + half_o;
-                const int o = row < len ? clamp127(x >> prm.sh_o) : 0;
-                w |= (static_cast<uint32_t>(o) & 0xffu) << (8 * e);
-            }
+            const uint32_t w = row < len ? out_word(oacc[2 * cc], oacc[2 * cc + 1], rr, prm.m_o, prm.sh_o) : 0u;
             *reinterpret_cast<uint32_t *>(prm.out + out_offset(prm, it.b, it.h, row) + 4 * t4 +
                                           16 * cc) = w;
         }
