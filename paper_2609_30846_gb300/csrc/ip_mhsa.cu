@@ -323,7 +323,12 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     prm.stall_injection = g_stall_injection;
     const int slots = resident_ctas(gs, smem);
     if (slots < 1) return IP_ERR_CUDA;
-    const ItemPlan ip = plan_items(N, slots);
+    ItemPlan ip = plan_items(N, slots);
+    // With a mask the live tiles are planned on the device, unless all of them
+    // are split in quarters anyway or every utterance is one tile.
+    prm.live_plan = lengths && B <= 32 && ntiles > 1 && g_split_mode < 0 && 4 * N > slots ? 1 : 0;
+    if (prm.live_plan) ip.grid = static_cast<uint32_t>(slots);
+    prm.grid_magic = iph::div_magic(ip.grid);
     prm.ntiles = ntiles;
     prm.tiles_magic = iph::div_magic(static_cast<unsigned long long>(ntiles));
     prm.heads_magic = iph::div_magic(static_cast<unsigned long long>(H));

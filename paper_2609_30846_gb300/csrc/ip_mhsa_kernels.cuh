@@ -79,7 +79,7 @@ __host__ __device__ inline SmemLayout smem_layout(int nchunk_max, bool global_sc
     L.remap = L.scores + (global_scores ? 0 : NCWARPS * nchunk_max * CHUNK_SCORE_BYTES);
     L.lut = L.remap + NCWARPS * REMAP_BYTES;
     L.bars = L.lut + LUT_ENTRIES * LUT_COPIES * 4;
-    L.total = L.bars + 128;
+    L.total = L.bars + 160;
     return L;
 }
 
@@ -101,13 +101,16 @@ struct FusedParams {
     // Work items, claimed in order by the persistent CTAs: items [0, nwhole)
     // are whole 64-row tiles in (b, h, tile) order, items [nwhole, nitems)
     // the 2^split_log2 parts (32-row halves or 16-row quarters) of the tiles
-    // from nwhole on.
+    // from nwhole on.  With live_plan (a key-padding mask) the items are those
+    // of LivePlan instead.
     unsigned int *sched;      // workspace words: [0] next item, [16] CTAs done claiming
     int ntiles;                        // 64-row tiles per (b, h)
     unsigned long long tiles_magic;    // udiv_magic constant of ntiles
     unsigned long long heads_magic;    // udiv_magic constant of H
     uint32_t nwhole, nitems;           // nitems < 2^31
     int split_log2;                    // 1: halves, 2: quarters
+    int live_plan;                     // plan over the live tiles (B <= 32)
+    unsigned long long grid_magic;     // udiv_magic constant of the grid (live_plan)
     int out_rows;             // output [B][T][H][DH] instead of [B][H][T][DH]
     uint8_t *gscores;         // global mode: score slices, NCWARPS per CTA, nchunk_max KB each
 };
@@ -448,7 +451,7 @@ __device__ __forceinline__ void prob_operand(const uint32_t (&pw)[4], uint32_t (
 }
 
 // Eq. 7 for the four outputs d = 16c + 4t .. + 3 of one row (byte e: n-tile 2c
-// + (e & 1), column 2t + (e >> 1)): |m_o acc| < 2^57 (acc < 255 127 T < 2^26), so
+// + (e & 1), column 2t + (e >> 1)).  |m_o acc| < 2^57 (acc < 255 128 T <= 2^26), so
 // the quotient by 2^31 is a 32-bit value; the upper clamp is the pack's.
 __device__ __forceinline__ uint32_t out_word(const int (&a)[4], const int (&b)[4], int rr, int m_o, int sh_o) {
     const long long rnd = 1ll << (sh_o - 1);
@@ -597,19 +600,13 @@ struct Item {
     bool pad;   // every row of the tile (half) is padding
 };
 
-__device__ __forceinline__ Item decode_item(const FusedParams &p, uint32_t item) {
+// Part `part` of 2^plog2 of tile `lin` in (b, h, tile) order (part -1, plog2
+// 0: the whole tile).
+__device__ __forceinline__ Item decode_item(const FusedParams &p, uint32_t lin, int part, int plog2) {
     Item it;
-    uint32_t lin = item;
-    it.part = -1;
-    it.nparts = 1;
-    it.plog2 = 0;
-    if (item >= p.nwhole) {
-        const uint32_t t = item - p.nwhole;
-        lin = p.nwhole + (t >> p.split_log2);
-        it.part = static_cast<int>(t & ((1u << p.split_log2) - 1u));
-        it.nparts = 1 << p.split_log2;
-        it.plog2 = p.split_log2;
-    }
+    it.part = part;
+    it.nparts = 1 << plog2;
+    it.plog2 = plog2;
     const uint32_t bh = udiv_magic(lin, p.tiles_magic);
     const int tile = static_cast<int>(lin - bh * static_cast<uint32_t>(p.ntiles));
     it.b = static_cast<int>(udiv_magic(bh, p.heads_magic));
@@ -625,6 +622,104 @@ __device__ __forceinline__ Item decode_item(const FusedParams &p, uint32_t item)
     it.nchunks = (len + NK - 1) / NK;
     it.pad = (it.part < 0 ? it.i0 : it.i0 + (MROWS >> it.plog2) * it.part) >= len;
     return it;
+}
+
+// The part and its log2 count as one word, beside the tile number in a slot.
+__device__ __forceinline__ uint32_t item_code(const Item &it) {
+    return static_cast<uint32_t>(it.part & 0xff) | (static_cast<uint32_t>(it.plog2) << 8);
+}
+__device__ __forceinline__ Item decode_slot(const FusedParams &p, uint32_t lin, uint32_t code) {
+    const int plog2 = static_cast<int>(code >> 8);
+    return decode_item(p, lin, plog2 ? static_cast<int>(code & 0xffu) : -1, plog2);
+}
+
+// Items of a batch with key padding, planned by every CTA's copy warp alike
+// from the lengths (one utterance per lane): the live 64-row tiles come first,
+// the longest utterances' before the shorter ones' (an item's cost goes with
+// its utterance's length), then the padding tiles, which only get zeros.  The
+// live tiles of a partial last round are split like a full batch's
+// (plan_items on the host counts padding as work).  At B = 16, T = 250 with
+// lengths in T/2 .. T about 440 of 512 tiles are live: a plan over all of them
+// left 208 for the second round of 304 and split none (61 us; 50 us planned so).
+struct LivePlan {
+    uint32_t nwhole, nlive, ntotal;   // whole items, live items, all items
+    int split_log2;
+    int b, nt;                        // this lane's utterance in order of length, its live tiles
+    uint32_t off, poff;               // live and padding tiles of the utterances before it
+};
+
+__device__ __forceinline__ uint32_t warp_exclusive_sum(uint32_t v, int lane, uint32_t &total) {
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    total = __shfl_sync(0xffffffffu, x, 31);
+    return x - v;
+}
+
+__device__ __forceinline__ LivePlan live_plan(const FusedParams &p, int lane) {
+    LivePlan L;
+    int len = -1;
+    if (lane < p.B) {
+        len = p.lengths[lane];
+        len = len < 0 ? 0 : (len > p.T ? p.T : len);
+    }
+    int rank = 0;
+    for (int j = 0; j < 32; ++j) {
+        const int o = __shfl_sync(0xffffffffu, len, j);
+        rank += o > len || (o == len && j < lane) ? 1 : 0;
+    }
+    L.b = 0;
+    for (int j = 0; j < 32; ++j)
+        if (__shfl_sync(0xffffffffu, rank, j) == lane) L.b = j;
+    len = __shfl_sync(0xffffffffu, len, L.b);
+    const bool real = lane < p.B;   // padding lanes (length -1) rank last
+    L.nt = real ? (len + MROWS - 1) / MROWS : 0;
+    uint32_t live, pads;
+    L.off = warp_exclusive_sum(static_cast<uint32_t>(L.nt) * p.H, lane, live);
+    L.poff = warp_exclusive_sum(real ? static_cast<uint32_t>(p.ntiles - L.nt) * p.H : 0u, lane, pads);
+    const uint32_t r = live - udiv_magic(live, p.grid_magic) * gridDim.x;   // tiles of the last round
+    L.split_log2 = 4 * r <= gridDim.x ? 2 : (2 * r <= gridDim.x ? 1 : 0);
+    L.nwhole = live - (L.split_log2 ? r : 0u);
+    L.nlive = L.nwhole + ((live - L.nwhole) << L.split_log2);
+    L.ntotal = L.nlive + pads;
+    return L;
+}
+
+// Item `item` of the plan (item < ntotal).
+__device__ __forceinline__ Item plan_item(const FusedParams &p, const LivePlan &L, uint32_t item, uint32_t &lin) {
+    const bool pad = item >= L.nlive;
+    int part = -1, plog2 = 0;
+    uint32_t i = item;
+    if (pad) {
+        i = item - L.nlive;
+    } else if (item >= L.nwhole) {
+        const uint32_t t = item - L.nwhole;
+        i = L.nwhole + (t >> L.split_log2);
+        part = static_cast<int>(t & ((1u << L.split_log2) - 1u));
+        plog2 = L.split_log2;
+    }
+    // the utterance that holds tile i: the last one that begins at or before it
+    const uint32_t first = pad ? L.poff : L.off;
+    const int at = __popc(__ballot_sync(0xffffffffu, first <= i)) - 1;
+    const uint32_t local = i - __shfl_sync(0xffffffffu, first, at);
+    const int b = __shfl_sync(0xffffffffu, L.b, at), nt = __shfl_sync(0xffffffffu, L.nt, at);
+    const uint32_t row = udiv_magic(local, p.heads_magic);   // tile-major within the utterance
+    const uint32_t h = local - row * static_cast<uint32_t>(p.H);
+    const uint32_t tile = row + (pad ? static_cast<uint32_t>(nt) : 0u);
+    lin = (static_cast<uint32_t>(b) * p.H + h) * static_cast<uint32_t>(p.ntiles) + tile;
+    return decode_item(p, lin, part, plog2);
+}
+
+// Item `item` of the host's plan (item < nitems).
+__device__ __forceinline__ Item host_item(const FusedParams &p, uint32_t item, uint32_t &lin) {
+    lin = item;
+    if (item < p.nwhole) return decode_item(p, lin, -1, 0);
+    const uint32_t t = item - p.nwhole;
+    lin = p.nwhole + (t >> p.split_log2);
+    return decode_item(p, lin, static_cast<int>(t & ((1u << p.split_log2) - 1u)), p.split_log2);
 }
 
 // Q fragments (A operand) of 16-row strip `strip` of the staged Q tile for
@@ -658,9 +753,10 @@ struct Ring {
     __device__ __forceinline__ uint32_t qtile() const { return stage_base + NSTAGE * STAGE_BYTES; }
     __device__ __forceinline__ uint32_t qfull() const { return bar_base + 8u * (3 * NSTAGE + 3); }
     __device__ __forceinline__ uint32_t qempty() const { return bar_base + 8u * (3 * NSTAGE + 4); }
-    // Item number of the CTA's live item k (written by the copy warp before
-    // it arrives on that item's barriers), or NO_ITEM after the last.
-    __device__ __forceinline__ uint32_t slot(int k) const { return bar_base + 96u + 4u * (k & 3); }
+    // The CTA's live item k: tile number and part (item_code), written by the
+    // copy warp before it arrives on that item's barriers, or NO_ITEM after the
+    // last.
+    __device__ __forceinline__ uint32_t slot(int k) const { return bar_base + 128u + 8u * (k & 3); }
     // The four consumer warps of a quarter item exchange maxima, sums and
     // partial sums (one phase per exchange step).
     __device__ __forceinline__ uint32_t quad() const { return bar_base + 120u; }
@@ -1418,22 +1514,31 @@ __global__ void __launch_bounds__(NTHREADS, 2)
     Item iss{};
     int iss_pos = 0, issued = 0;
     int kq = 0;   // live items published (slots written, Q tiles sent)
-    auto claim = [&](uint32_t &item) -> bool {
+    LivePlan plan{};
+    bool first_claim = true;
+    auto claim = [&](uint32_t &lin) -> bool {
+        const uint32_t n = prm.live_plan ? plan.ntotal : prm.nitems;
         for (;;) {
-            uint32_t x = 0;
-            if (lane == 0) x = atomicAdd(prm.sched, 1u);
-            item = __shfl_sync(0xffffffffu, x, 0);
-            if (item >= prm.nitems) return false;
-            iss = decode_item(prm, item);
+            // one round or less: the first item is the block's, without the
+            // round trip to the counter (0.2 us of a 7.9 us call)
+            uint32_t item = blockIdx.x;
+            if (!first_claim || n > gridDim.x) {
+                uint32_t x = 0;
+                if (lane == 0) x = atomicAdd(prm.sched, 1u);
+                item = __shfl_sync(0xffffffffu, x, 0) + (n > gridDim.x ? 0u : gridDim.x);
+            }
+            first_claim = false;
+            if (item >= n) return false;
+            iss = prm.live_plan ? plan_item(prm, plan, item, lin) : host_item(prm, item, lin);
             if (!iss.pad) return true;
             zero_rows(prm, iss, lane);
         }
     };
     // Publishes the claimed item as live item kq: its slot, then its Q tile
     // (the arrive on qfull releases the slot write).
-    auto publish = [&](uint32_t item) {
+    auto publish = [&](uint32_t lin) {
         if (lane == 0) {
-            sts32(R.slot(kq), item);
+            sts64(R.slot(kq), static_cast<int>(lin), static_cast<int>(item_code(iss)));
             mbar_expect_tx(R.qfull(), Q_TILE_BYTES);
             tma_load_3d(R.qtile(), &tm_q, 0, iss.i0, iss.bh, R.qfull());
         }
@@ -1485,10 +1590,11 @@ __global__ void __launch_bounds__(NTHREADS, 2)
         }
         __syncwarp();
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        uint32_t item = 0;
-        live0 = claim(item);
+        if (prm.live_plan) plan = live_plan(prm, lane);
+        uint32_t lin = 0;
+        live0 = claim(lin);
         if (live0) {
-            publish(item);
+            publish(lin);
             for (int u = 0; u < NSTAGE; ++u) {   // an item has at least two uses
                 if (lane == 0) issue(iss, iss_pos, u);
                 ++iss_pos;
@@ -1499,10 +1605,12 @@ __global__ void __launch_bounds__(NTHREADS, 2)
             done_claiming();
         }
     }
-    for (int d = threadIdx.x; d < LUT_ENTRIES; d += NTHREADS) {
-        const uint32_t e = iexp_neg(d, prm.q_ln2, prm.q_b, prm.q_c, prm.ln2_magic);
+    if (warp != NCWARPS) {   // the copy warp's first item and copies come first
+        for (int d = threadIdx.x - (warp > NCWARPS ? 32 : 0); d < LUT_ENTRIES; d += NTHREADS - 32) {
+            const uint32_t e = iexp_neg(d, prm.q_ln2, prm.q_b, prm.q_c, prm.ln2_magic);
 #pragma unroll
-        for (int c = 0; c < LUT_COPIES; ++c) sts32(lut + (d * LUT_COPIES + c) * 4, e);
+            for (int c = 0; c < LUT_COPIES; ++c) sts32(lut + (d * LUT_COPIES + c) * 4, e);
+        }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
@@ -1529,12 +1637,12 @@ __global__ void __launch_bounds__(NTHREADS, 2)
                     ok = false;
                     break;
                 }
-                uint32_t item = 0;
-                if (!claim(item)) {
+                uint32_t lin = 0;
+                if (!claim(lin)) {
                     finish(u + 2);
                     break;
                 }
-                publish(item);
+                publish(lin);
             }
             if (lane == 0) issue(iss, iss_pos, u + 2);
             ++iss_pos;
@@ -1563,9 +1671,9 @@ __global__ void __launch_bounds__(NTHREADS, 2)
                 if (lane == 0) atomicOr(prm.err, ERR_TIMEOUT_FULL);
                 return;
             }
-            const uint32_t item = lds32(R.slot(kb));
-            if (item == NO_ITEM) return;
-            const Item it = decode_item(prm, item);
+            const int2 item = lds64(R.slot(kb));
+            if (static_cast<uint32_t>(item.x) == NO_ITEM) return;
+            const Item it = decode_slot(prm, static_cast<uint32_t>(item.x), static_cast<uint32_t>(item.y));
             if (it.h != cur_h) {
                 cur_h = it.h;
                 const uint4 *u4 = reinterpret_cast<const uint4 *>(prm.u + static_cast<size_t>(cur_h) * DH);
@@ -1607,9 +1715,9 @@ __global__ void __launch_bounds__(NTHREADS, 2)
             if (lane == 0) atomicOr(prm.err, ERR_TIMEOUT_FULL);
             return;
         }
-        const uint32_t item = lds32(R.slot(k));
-        if (item == NO_ITEM) return;
-        const Item it = decode_item(prm, item);
+        const int2 item = lds64(R.slot(k));
+        if (static_cast<uint32_t>(item.x) == NO_ITEM) return;
+        const Item it = decode_slot(prm, static_cast<uint32_t>(item.x), static_cast<uint32_t>(item.y));
         const bool ok =
             it.nparts == 1   ? consume_whole<GS>(prm, it, u0, R, remap, scores, lut, warp, lane)
             : it.nparts == 2 ? consume_half<GS>(prm, it, u0, R, remap, scores, lut, pair_bar(warp >> 1),
