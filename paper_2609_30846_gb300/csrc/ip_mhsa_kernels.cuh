@@ -450,22 +450,29 @@ __device__ __forceinline__ void prob_operand(const uint32_t (&pw)[4], uint32_t (
     af[3] = __byte_perm(pw[2], pw[3], 0x7632);
 }
 
-// Eq. 7 for the four outputs d = 16c + 4t .. + 3 of one row (byte e: n-tile 2c
-// + (e & 1), column 2t + (e >> 1)).  |m_o acc| < 2^57 (acc < 255 128 T <= 2^26), so
-// the quotient by 2^31 is a 32-bit value; the upper clamp is the pack's.
-__device__ __forceinline__ uint32_t out_word(const int (&a)[4], const int (&b)[4], int rr, int m_o, int sh_o) {
+// Eq. 7 for the outputs of d chunk c (n-tiles 2c and 2c + 1: a thread's columns
+// 2t, 2t + 1 of both) and rows g, g + 8 in one word each.  |m_o acc| < 2^57
+// (acc < 255 128 T <= 2^26), so the quotient by 2^31 is a 32-bit value; the upper
+// clamp is the pack's.  Threads 2t' and 2t' + 1 exchange one half each: the even
+// one ends with d = 16c + 4t' .. + 3, the odd one with the same + 8 (out_col).
+__device__ __forceinline__ void out_words(const int (&a)[4], const int (&b)[4], int m_o, int sh_o, int t4,
+                                          uint32_t (&w)[2]) {
     const long long rnd = 1ll << (sh_o - 1);
-    const int acc[4] = {a[2 * rr], b[2 * rr], a[2 * rr + 1], b[2 * rr + 1]};
-    int z[4];
+    int z[8];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const long long x = static_cast<long long>(m_o) * acc[e] + rnd;
+    for (int e = 0; e < 8; ++e) {
+        const long long x = static_cast<long long>(m_o) * (e < 4 ? a[e] : b[e - 4]) + rnd;
         z[e] = max(static_cast<int>(__funnelshift_r(static_cast<uint32_t>(x), static_cast<uint32_t>(x >> 32), 31)) >>
                        (sh_o - 31),
                    -127);
     }
-    return pack_sat4(z[0], z[1], z[2], z[3]);
+    const uint32_t wa = pack_sat4(z[0], z[1], z[2], z[3]), wb = pack_sat4(z[4], z[5], z[6], z[7]);
+    const uint32_t got = __shfl_xor_sync(0xffffffffu, (t4 & 1) ? wa : wb, 1);
+    const uint32_t lo = (t4 & 1) ? got : wa, hi = (t4 & 1) ? wb : got;
+    w[0] = __byte_perm(lo, hi, 0x5410);
+    w[1] = __byte_perm(lo, hi, 0x7632);
 }
+__device__ __forceinline__ int out_col(int t4) { return 8 * (t4 & 1) + 4 * (t4 >> 1); }
 
 // ------------------------------------------------------- split-tile parts --
 // In a split tile the two warps of a row strip take the key halves
@@ -549,14 +556,15 @@ __device__ __forceinline__ void finish_half(int (&oacc)[16][4], uint32_t pxo, in
         for (int e = 0; e < 4; ++e)
             oacc[8 * HK + i][e] += static_cast<int>(lds32(pxo + ((i * 4 + e) * 32 + lane) * 4));
 #pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-        const int row = wrow0 + g + 8 * rr;
-        if (row >= T) continue;
-        int8_t *dst = prm.out + out_offset(prm, b, h, row) + 4 * t4;
+    for (int c = 4 * HK; c < 4 * HK + 4; ++c) {
+        uint32_t w[2];
+        out_words(oacc[2 * c], oacc[2 * c + 1], prm.m_o, prm.sh_o, t4, w);
 #pragma unroll
-        for (int c = 4 * HK; c < 4 * HK + 4; ++c) {
-            *reinterpret_cast<uint32_t *>(dst + 16 * c) =
-                row < len ? out_word(oacc[2 * c], oacc[2 * c + 1], rr, prm.m_o, prm.sh_o) : 0u;
+        for (int rr = 0; rr < 2; ++rr) {
+            const int row = wrow0 + g + 8 * rr;
+            if (row < T)
+                *reinterpret_cast<uint32_t *>(prm.out + out_offset(prm, b, h, row) + out_col(t4) + 16 * c) =
+                    row < len ? w[rr] : 0u;
         }
     }
 }
@@ -1001,15 +1009,16 @@ __device__ __forceinline__ bool consume_whole(const FusedParams &prm, const Item
     // d = 16c + 4t .. 16c + 4t + 3 (n-tiles 2c, 2c + 1, columns 2t, 2t + 1).
     // The d chunks go in the order their last MMAs were issued, so the
     // first ones are requantised while the pipe finishes the others.
+    int8_t *const dst0 = prm.out + out_offset(prm, it.b, it.h, wrow0 + g) + out_col(t4);
+    const size_t row8 = 8 * static_cast<size_t>(prm.out_rows ? prm.H : 1) * DH;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
+        uint32_t w[2];
+        out_words(oacc[2 * c], oacc[2 * c + 1], prm.m_o, prm.sh_o, t4, w);
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
             const int row = wrow0 + g + 8 * rr;
-            const uint32_t w = row < len ? out_word(oacc[2 * c], oacc[2 * c + 1], rr, prm.m_o, prm.sh_o) : 0u;
-            if (row < T)
-                *reinterpret_cast<uint32_t *>(prm.out + out_offset(prm, it.b, it.h, row) + 4 * t4 +
-                                              16 * c) = w;
+            if (row < T) *reinterpret_cast<uint32_t *>(dst0 + rr * row8 + 16 * c) = row < len ? w[rr] : 0u;
         }
     }
     return true;
@@ -1372,7 +1381,7 @@ __device__ __forceinline__ bool consume_quarter(const FusedParams &prm, const It
     int oacc[16][4];
 #pragma unroll
     for (int nt = 0; nt < 16; ++nt) oacc[nt][0] = oacc[nt][1] = oacc[nt][2] = oacc[nt][3] = 0;
-    const int vkey = 16 * warp + 8 * ((lane >> 3) & 1) + (lane & 7);
+    const int vkey = 16 * warp + vkey16(lane);
     for (int c = 0; c < nchunks; ++c) {
         const int kvalid = len - c * NK - 16 * warp;
         const int2 wv = sc_ld64<GS>(scores, c * CHUNK_SCORE_BYTES + lane * 8);
@@ -1393,13 +1402,13 @@ __device__ __forceinline__ bool consume_quarter(const FusedParams &prm, const It
         const uint32_t vtile = R.stage(u);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            // d chunks 2j, 2j + 1: the slice's keys 0-7 and 8-15 of each
+            // d chunks 2j (lanes 0-15's addresses) and 2j + 1 of the slice's keys
             uint32_t r0, r1, r2, r3;
-            ldsm_x4_trans(vtile + swz(vkey, 2 * j + (lane >> 4)), r0, r1, r2, r3);
-            mma_u8s8_k16(oacc[4 * j], a0, a1, __byte_perm(r0, r1, 0x6420));
-            mma_u8s8_k16(oacc[4 * j + 1], a0, a1, __byte_perm(r0, r1, 0x7531));
-            mma_u8s8_k16(oacc[4 * j + 2], a0, a1, __byte_perm(r2, r3, 0x6420));
-            mma_u8s8_k16(oacc[4 * j + 3], a0, a1, __byte_perm(r2, r3, 0x7531));
+            ldsm_x2_trans_b8(vtile + swz(vkey, 2 * j + (lane >> 4)), r0, r1, r2, r3);
+            mma_u8s8_k16(oacc[4 * j], a0, a1, r0);
+            mma_u8s8_k16(oacc[4 * j + 1], a0, a1, r1);
+            mma_u8s8_k16(oacc[4 * j + 2], a0, a1, r2);
+            mma_u8s8_k16(oacc[4 * j + 3], a0, a1, r3);
         }
         release_stage(R.empty(u), lane);
     }
@@ -1439,13 +1448,14 @@ __device__ __forceinline__ bool consume_quarter(const FusedParams &prm, const It
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
         if ((cc >> 1) != warp) continue;
+        uint32_t w[2];
+        out_words(oacc[2 * cc], oacc[2 * cc + 1], prm.m_o, prm.sh_o, t4, w);
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
             const int row = wrow0 + g + 8 * rr;
-            if (row >= T) continue;
-            const uint32_t w = row < len ? out_word(oacc[2 * cc], oacc[2 * cc + 1], rr, prm.m_o, prm.sh_o) : 0u;
-            *reinterpret_cast<uint32_t *>(prm.out + out_offset(prm, it.b, it.h, row) + 4 * t4 +
-                                          16 * cc) = w;
+            if (row < T)
+                *reinterpret_cast<uint32_t *>(prm.out + out_offset(prm, it.b, it.h, row) + out_col(t4) + 16 * cc) =
+                    row < len ? w[rr] : 0u;
         }
     }
     return true;

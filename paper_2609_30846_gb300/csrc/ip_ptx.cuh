@@ -113,11 +113,12 @@ __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t &r0, uint32_t &r
                  : "r"(addr));
 }
 
-// Four 8x8 matrices of 16-bit elements, transposed: thread l receives, of
-// matrix i, the elements (2 (l & 3), l >> 2) and (2 (l & 3) + 1, l >> 2).
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1,
-                                              uint32_t &r2, uint32_t &r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+// Two 16x16 matrices of bytes, transposed (rows of matrix i at the addresses of
+// lanes 16 i .. 16 i + 15): thread l receives, of matrix i, the elements of rows
+// 4 (l & 3) .. + 3 in column l >> 2 (first register) and in column 8 + (l >> 2).
+__device__ __forceinline__ void ldsm_x2_trans_b8(uint32_t addr, uint32_t &r0, uint32_t &r1,
+                                                 uint32_t &r2, uint32_t &r3) {
+    asm volatile("ldmatrix.sync.aligned.m16n16.x2.trans.shared.b8 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                  : "r"(addr));
 }
