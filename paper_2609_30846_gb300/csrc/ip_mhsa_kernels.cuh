@@ -1,7 +1,8 @@
 // Device code of the integer-only relative-positional MHSA (I-Parakeet,
 // Sec. 3.1) for sm_103a.  Integer arithmetic only: no floating-point type
 // appears in this file, and no division by a run-time value (the two
-// divisions the method needs are done by binary long division).
+// divisions the method needs are multiplications: a Newton reciprocal and an
+// exact multiply-high).
 //
 // sm_103a has no integer tcgen05 MMA kind, so the three contractions use the
 // integer warp MMA (mma.sync m16n8k32, s8 x s8 and u8 x s8 -> s32, which
@@ -206,43 +207,60 @@ __device__ __forceinline__ uint32_t lut_at(uint32_t lut_g, uint32_t d4, int e) {
     return lut_g + ((d4 >> (8 * e)) & 0xffu) * (LUT_COPIES * 4);
 }
 
-// B fragments of the attn.V MMA for keys 32 ks .. 32 ks + 31 of the staged
-// V tile (keys as rows, 128-byte swizzle) and the 16 values of d in chunk c,
-// with no transposed copy of V: ldmatrix.trans on 16-bit elements hands
-// thread (g, t) the byte pairs (d = 16c + 2g, 16c + 2g + 1) of keys 2t, 2t + 1
-// (r0), 8 + 2t, 9 + 2t (r1) and the same + 16 (r2, r3); byte selects split
-// them into the fragment of the even d (n-tile 2c) and of the odd d (n-tile
-// 2c + 1).  The k order, keys 2t, 2t + 1, 8 + 2t, 9 + 2t then + 16, is the one
-// of the probability operand (prob_operand).  N-tile 2c + p holds d =
-// 16c + 2n + p in its column n.
-__device__ __forceinline__ void vfrag(uint32_t vtile, int ks, int c, int lane, uint32_t &b0e,
-                                      uint32_t &b1e, uint32_t &b0o, uint32_t &b1o) {
-    const int key = 32 * ks + 8 * (lane >> 3) + (lane & 7);
-    uint32_t r0, r1, r2, r3;
-    ldsm_x4_trans(vtile + swz(key, c), r0, r1, r2, r3);
-    b0e = __byte_perm(r0, r1, 0x6420);
-    b1e = __byte_perm(r2, r3, 0x6420);
-    b0o = __byte_perm(r0, r1, 0x7531);
-    b1o = __byte_perm(r2, r3, 0x7531);
+// Key (0 .. 15) that lane i supplies to the 8-bit transposing ldmatrix: thread
+// (g, t) receives the keys 2t, 2t + 1, 8 + 2t, 9 + 2t in one register, the k
+// order of the probability operand (prob_operand).
+__device__ __forceinline__ int vkey16(int lane) {
+    return 2 * ((lane >> 2) & 3) + (lane & 1) + 4 * (lane & 2);
 }
 
-// floor(2^32 / s) for s >= 2 by restoring binary long division (the
-// quotient is at most 2^31).  With 2^(L-1) <= s < 2^L the quotient is at
-// most 2^(33-L), so the digits start at bit 33 - L.
-__device__ __forceinline__ uint32_t div_2pow32(unsigned long long s) {
-    if (s > (1ull << 32)) return 0u;
-    unsigned long long rem = 1ull << 32;
-    uint32_t quo = 0;
-    const int top = __clzll(static_cast<long long>(s)) - 31;   // 33 - L
-#pragma unroll 1
-    for (int bit = top < 31 ? top : 31; bit >= 0; --bit) {
-        const unsigned long long t = s << bit;
-        if (t <= rem) {
-            rem -= t;
-            quo |= 1u << bit;
-        }
+// B fragments of the attn.V MMA for keys 32 ks .. 32 ks + 31 of the staged
+// V tile (keys as rows, 128-byte swizzle) and the 16 values of d in chunk c,
+// with no transposed copy of V and no byte selects (an ldmatrix on 16-bit
+// pairs and four selects per fragment pair before): n-tile 2c holds d =
+// 16c .. 16c + 7, n-tile 2c + 1 the next eight.
+__device__ __forceinline__ void vfrag(uint32_t vtile, int ks, int c, int lane, uint32_t &b0a,
+                                      uint32_t &b1a, uint32_t &b0b, uint32_t &b1b) {
+    const int key = 32 * ks + 16 * (lane >> 4) + vkey16(lane);
+    ldsm_x2_trans_b8(vtile + swz(key, c), b0a, b0b, b1a, b1b);
+}
+
+// floor(2^32 / s) for s >= 2 by Newton's iteration on the reciprocal of the
+// normalised divisor, with 32-bit multiplications.  With X = s 2^L / 2^32 in
+// [1/2, 1) (L leading zeros), r approximates 2^31 / X: it starts from 2^31 (48 -
+// 32 X) / 17 (relative error at most 1/17), and each step r <- r (2 - X r) squares
+// the error (three steps: below 2^-29 with the truncations).  floor(2^32 / s) is
+// then r 2^(L - 31) to within two, and the remainder 2^32 - q s settles it.
+// About 35 instructions in a short chain; the binary long division before took
+// ten for each bit of the quotient, between the exponential sums and the first
+// probabilities of every item.
+__device__ __forceinline__ uint32_t div_2pow32(unsigned long long s64) {
+    if (s64 >> 32) return s64 == (1ull << 32) ? 1u : 0u;
+    const uint32_t s = static_cast<uint32_t>(s64);
+    const int L = __clz(static_cast<int>(s));
+    const uint32_t x = s << L;
+    uint32_t r = 1768515945u - __umulhi(x, 4042322161u);   // modulo 2^32
+#pragma unroll
+    for (int it = 0; it < 3; ++it) {
+        const uint32_t t = __umulhi(x, r);                 // 2^31 X r
+        const unsigned long long p = static_cast<unsigned long long>(r) * (0u - t);
+        r = __funnelshift_r(static_cast<uint32_t>(p), static_cast<uint32_t>(p >> 32), 31);
     }
-    return quo;
+    uint32_t q = r >> (31 - L);
+    long long rem = (1ll << 32) - static_cast<long long>(static_cast<unsigned long long>(q) * s);
+#pragma unroll
+    for (int it = 0; it < 2; ++it)
+        if (rem < 0) {
+            --q;
+            rem += s;
+        }
+#pragma unroll
+    for (int it = 0; it < 2; ++it)
+        if (rem >= static_cast<long long>(s)) {
+            ++q;
+            rem -= s;
+        }
+    return q;
 }
 
 // I-BERT integer exponential of d = -nd (0 <= nd < 512): z = floor(nd /
