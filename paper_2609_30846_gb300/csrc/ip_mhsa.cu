@@ -147,13 +147,16 @@ int ensure_smem(bool gs, int bytes) {
 // CTAs an SM holds at this shared-memory size), cached for the last query
 // of each form.
 std::mutex g_occ_mu;
-int g_occ_dev[2] = {-1, -1}, g_occ_smem[2] = {-1, -1}, g_occ_slots[2] = {0, 0};
+int g_occ_dev[2] = {-1, -1}, g_occ_smem[2] = {-1, -1}, g_occ_slots[2] = {0, 0}, g_occ_sms[2] = {0, 0};
 
-int resident_ctas(bool gs, int smem) {
+int resident_ctas(bool gs, int smem, int *sms = nullptr) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lock(g_occ_mu);
-    if (dev == g_occ_dev[gs] && smem == g_occ_smem[gs]) return g_occ_slots[gs];
+    if (dev == g_occ_dev[gs] && smem == g_occ_smem[gs]) {
+        if (sms) *sms = g_occ_sms[gs];
+        return g_occ_slots[gs];
+    }
     int nsm = 0, per_sm = 0;
     if (ensure_smem(gs, smem) != IP_OK ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -163,6 +166,8 @@ int resident_ctas(bool gs, int smem) {
     g_occ_dev[gs] = dev;
     g_occ_smem[gs] = smem;
     g_occ_slots[gs] = nsm * per_sm;
+    g_occ_sms[gs] = nsm;
+    if (sms) *sms = nsm;
     return g_occ_slots[gs];
 }
 
@@ -170,6 +175,8 @@ int resident_ctas(bool gs, int smem) {
 // has room: the shared-memory slices of T <= 384 (6 chunks) let two CTAs
 // share an SM, longer ones only one.
 constexpr int GS_MIN_T = 6 * ipk::NK + 1;
+
+constexpr int OWN_SM_SMEM = 120 * 1024;   // more than half of an SM's
 
 int fused_smem(int T, bool gs) {
     return ipk::smem_layout((T + ipk::NK - 1) / ipk::NK, gs).total + 1024;
@@ -321,7 +328,8 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     prm.f24 = !g_wide_sums && e0 > 256ull ? 1 : 0;
     prm.timeout_cycles = g_timeout_cycles;
     prm.stall_injection = g_stall_injection;
-    const int slots = resident_ctas(gs, smem);
+    int sms = 0;
+    const int slots = resident_ctas(gs, smem, &sms);
     if (slots < 1) return IP_ERR_CUDA;
     ItemPlan ip = plan_items(N, slots);
     // With a mask the live tiles are planned on the device, unless all of them
@@ -332,6 +340,12 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     prm.ntiles = ntiles;
     prm.tiles_magic = iph::div_magic(static_cast<unsigned long long>(ntiles));
     prm.heads_magic = iph::div_magic(static_cast<unsigned long long>(H));
+    // No more CTAs than SMs: each takes an SM of its own, also where the launch
+    // before still holds some of them (two would share one and run slower: B = 1,
+    // T = 250 17.0 us, 14.2 us so).
+    const int own = ip.grid <= static_cast<uint32_t>(sms) && smem < OWN_SM_SMEM ? OWN_SM_SMEM : smem;
+    rc = ensure_smem(gs, own);
+    if (rc != IP_OK) return rc;
     prm.nwhole = ip.nwhole;
     prm.split_log2 = ip.split_log2;
     prm.nitems = ip.nitems;
@@ -341,7 +355,7 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     // kernel before it on the stream finishes (the kernel waits for that
     // grid before its first global access, so the order of the two is kept).
     if (iph::launch_pdl(fused_kernel(gs), dim3(ip.grid), dim3(ipk::NTHREADS),
-                        static_cast<size_t>(smem), st, tm_q, tm_k, tm_v, tm_p, prm) != cudaSuccess)
+                        static_cast<size_t>(own), st, tm_q, tm_k, tm_v, tm_p, prm) != cudaSuccess)
         return IP_ERR_CUDA;
     if (cudaGetLastError() != cudaSuccess) return IP_ERR_CUDA;
     return IP_OK;
