@@ -29,6 +29,11 @@ int sm_count() {
     return g_sms[dev];
 }
 
+// Up to this many rows one CTA per row is the faster kernel (us, batched / row,
+// d = 512, 1024, 2048: 2.4 / 1.6, 2.8 / 2.0, 4.1 / 2.9 at 125 rows, 2.4 / 2.1, 2.8 /
+// 2.6, 4.1 / 4.1 at 250, 2.5 / 2.3, 2.8 / 4.1, 4.2 / 4.9 at 400).
+constexpr long long ROW_KERNEL_ROWS = 256;
+
 // CTAs of the C-segment kernel on the whole GPU: one per SM, so that its
 // eight warps take two or more batches each and load the next batch's rows
 // while they normalise the current one (cached; 0 if one does not fit).
@@ -41,7 +46,7 @@ long long resident(int nsm) {
     if (per_sm[dev] == 0) {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, ipn::layernorm_i8_kernel<C>,
-                                                          ipn::THREADS, C * 8192) != cudaSuccess ||
+                                                          ipn::THREADS, ipn::record_bytes(C)) != cudaSuccess ||
             n < 1)
             return 0;
         per_sm[dev] = 1;
@@ -51,12 +56,18 @@ long long resident(int nsm) {
 
 template <int C>
 int launch(const ipn::NormParams &prm, int nsm, cudaStream_t st) {
+    if (prm.rows <= ROW_KERNEL_ROWS) {
+        if (iph::launch_pdl(ipn::layernorm_row_kernel<C>, dim3(static_cast<unsigned>(prm.rows)),
+                            dim3(ipn::ROW_THREADS), 0, st, prm) != cudaSuccess)
+            return IP_ERR_CUDA;
+        return cudaGetLastError() == cudaSuccess ? IP_OK : IP_ERR_CUDA;
+    }
     // every resident CTA gets batches (dealt warp-major), up to one per CTA
     const long long batches = (prm.rows + ipn::NB - 1) / ipn::NB;
     const long long cap = resident<C>(nsm);
     if (cap <= 0) return IP_ERR_CUDA;
     const unsigned grid = static_cast<unsigned>(batches < cap ? batches : cap);
-    if (iph::launch_pdl(ipn::layernorm_i8_kernel<C>, dim3(grid), dim3(ipn::THREADS), C * 8192, st,
+    if (iph::launch_pdl(ipn::layernorm_i8_kernel<C>, dim3(grid), dim3(ipn::THREADS), ipn::record_bytes(C), st,
                         prm) != cudaSuccess)
         return IP_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? IP_OK : IP_ERR_CUDA;

@@ -6,8 +6,8 @@
 //
 // One warp per batch of four rows of d channels, batches dealt warp-major
 // over a grid of one CTA per SM, so that every warp takes two or more
-// batches and loads the next one's rows during the current pass B.  Per row: the sum and the sum of squares of the
-// int8 values (dp4a, warp reduction), floor(sum c^2 / d) = d sum q^2 -
+// batches and loads the next one's rows during the current pass B.  Per row:
+// the sum and the sum of squares of the int8 values (dp4a, warp reduction), floor(sum c^2 / d) = d sum q^2 -
 // (sum q)^2 exactly for the centred values c_i = d q_i - sum, sigma =
 // isqrt(that + eps_c) (at least 1), f = floor(2^31 / sigma), and per element
 // n = round(c f / 2^16), y = clamp(round((M_i n + B_i) / 2^E_i), -127, 127).
@@ -17,7 +17,13 @@
 // Lane l takes the 16-byte segments l, l + 32, ... of the row (coalesced)
 // and keeps them in registers between the two passes; the per-channel
 // constants (B, M, E) of its channels sit in shared memory in lane-major
-// order, one 16-byte record per channel, each read once per batch of rows.
+// order, one 16-byte record per channel, each read once per batch of rows.  What
+// bounds it: the dependency chain of an element (multiply-add, shift, 64-bit
+// multiply-add, shift, clamp, pack) with two warps per sub-partition, and for
+// few rows the set-up of the records (12000 x 1024: 9.8 -> 8.9 us with the
+// constants loaded at once and the records written without bank conflicts; 1332
+// x 1024 4.1 -> 2.9 us).  Few rows take layernorm_row_kernel (125 x 1024: 3.9 ->
+// 2.0 us).
 #pragma once
 
 #include <stdint.h>
@@ -31,6 +37,12 @@ using namespace ipk;
 constexpr int THREADS = 256;              // 8 warps, one batch of rows each
 constexpr int NB = 4;                     // rows per warp batch
 constexpr int ERR_PARAM = 16;             // a per-channel constant out of its domain
+
+// Place of the record of segment j, lane l, element e: a lane's sixteen records
+// together and one of padding, so that neither the lanes of a read (one e) nor
+// the threads that write consecutive channels meet on a bank.
+__host__ __device__ constexpr int record(int j, int l, int e) { return (j * 32 + l) * 17 + e; }
+constexpr int record_bytes(int C) { return C * 32 * 17 * 16; }
 
 struct NormParams {
     const int8_t *x;
@@ -100,6 +112,35 @@ __device__ __forceinline__ uint32_t recip_2pow31(unsigned long long s64) {
     return static_cast<uint32_t>(q);
 }
 
+// Factors of a row from the sum and the sum of squares of its int8 values: the
+// normalised value of element q is n = floor((q F + G) / 2^7).  sum c^2 / d is d
+// sum q^2 - (sum q)^2 exactly (c = d q - sum), sigma = max(1, isqrt(that + eps_c)),
+// f = floor(2^31 / sigma), held as a signed 32-bit value: f = 2^31 only for sigma
+// = 1, where sum c^2 < 4 d gives |c| < 2^7 and round(c (2^31 - 1) / 2^16) =
+// round(c 2^31 / 2^16), so 2^31 - 1 stands in exactly.
+// n = floor(u / 2^16) with u = c f + 2^15 and c = D q - sum, D = C 2^9: u = (q C f
+// + G) 2^9 + l with G = floor((2^15 - sum f) / 2^9) and 0 <= l < 2^9, so n =
+// floor((q C f + G) / 2^7) (the fraction l / 2^9 never carries an integer
+// quotient over).  With s = sqrt(sum c^2 / d + eps_c), sigma >= s / 2 when s >= 1
+// (and every c is 0 when s < 1), and |c| <= sqrt(d) s, so |c| f <= 2^32 sqrt(d)
+// and |q C f + G| < 2^29: the 32-bit multiply-add modulo 2^32 gives it exactly.
+template <int C>
+__device__ __forceinline__ uint32_t row_f(long long eps_c, int sum, int sq) {
+    const long long ms = 512ll * C * sq - static_cast<long long>(sum) * sum;
+    const unsigned long long sigma = isqrt_u42(static_cast<unsigned long long>(ms + eps_c));
+    const uint32_t f = recip_2pow31(sigma < 1 ? 1 : sigma);
+    return f > 0x7fffffffu ? 0x7fffffffu : f;
+}
+template <int C>
+__device__ __forceinline__ void row_factors_of(uint32_t f, int sum, uint32_t &F, uint32_t &G) {
+    F = static_cast<uint32_t>(C) * f;
+    G = static_cast<uint32_t>(((1ll << 15) - static_cast<long long>(sum) * static_cast<long long>(f)) >> 9);
+}
+template <int C>
+__device__ __forceinline__ void row_factors(long long eps_c, int sum, int sq, uint32_t &F, uint32_t &G) {
+    row_factors_of<C>(row_f<C>(eps_c, sum, sq), sum, F, G);
+}
+
 // C = d / 512 segments of 16 channels per lane.  A warp takes NB rows at a
 // time and keeps their int8 values in registers: it reduces them, lane r
 // computes the square root and the reciprocal of row r (one chain of those
@@ -114,7 +155,7 @@ __device__ __forceinline__ uint32_t recip_2pow31(unsigned long long s64) {
 template <int C>
 struct Batch {
     uint4 xv[NB][C];
-    uint32_t F[NB], G[NB];   // n = floor((q F + G) / 2^7) for row r (see pass_a)
+    uint32_t F[NB], G[NB];   // n = floor((q F + G) / 2^7) for row r (row_f)
 };
 
 template <int C>
@@ -133,7 +174,6 @@ __device__ __forceinline__ void load_rows(const NormParams &prm, long long row0,
 
 template <int C>
 __device__ __forceinline__ void pass_a_stats(const NormParams &prm, int lane, Batch<C> &bt) {
-    constexpr int D = 512 * C;
     int sq[NB], sum[NB];
 #pragma unroll
     for (int r = 0; r < NB; ++r) {
@@ -156,31 +196,17 @@ __device__ __forceinline__ void pass_a_stats(const NormParams &prm, int lane, Ba
             sum[r] += __shfl_xor_sync(0xffffffffu, sum[r], o);
             sq[r] += __shfl_xor_sync(0xffffffffu, sq[r], o);
         }
-    long long ms = 0;
+    int own_sum = 0, own_sq = 0;
 #pragma unroll
     for (int r = 0; r < NB; ++r)
-        if (lane == r) ms = static_cast<long long>(D) * sq[r] - static_cast<long long>(sum[r]) * sum[r];
-    unsigned long long sigma = isqrt_u42(static_cast<unsigned long long>(ms + prm.eps_c));
-    sigma = sigma < 1 ? 1 : sigma;
-    // f = floor(2^31 / sigma), held as a signed 32-bit value: f = 2^31 only
-    // for sigma = 1, where sum c^2 < 4 d gives |c| < 2^7 and round(c (2^31 -
-    // 1) / 2^16) = round(c 2^31 / 2^16), so 2^31 - 1 stands in exactly
-    uint32_t f_own = recip_2pow31(sigma);
-    f_own = f_own > 0x7fffffffu ? 0x7fffffffu : f_own;
-    // n = floor(u / 2^16) with u = c f + 2^15 and c = D q - sum, D = C 2^9:
-    // u = (q C f + G) 2^9 + l with G = floor((2^15 - sum f) / 2^9) and
-    // 0 <= l < 2^9, so n = floor((q C f + G) / 2^7) (the fraction l / 2^9
-    // never carries an integer quotient over).  With s = sqrt(sum c^2 / d +
-    // eps_c), sigma >= s / 2 when s >= 1 (and every c is 0 when s < 1), and
-    // |c| <= sqrt(d) s, so |c| f <= 2^32 sqrt(d) and |q C f + G| < 2^29:
-    // the 32-bit multiply-add modulo 2^32 gives it exactly.
+        if (lane == r) {
+            own_sum = sum[r];
+            own_sq = sq[r];
+        }
+    const uint32_t f_own = row_f<C>(prm.eps_c, own_sum, own_sq);
 #pragma unroll
-    for (int r = 0; r < NB; ++r) {
-        const uint32_t f = __shfl_sync(0xffffffffu, f_own, r);
-        bt.F[r] = static_cast<uint32_t>(C) * f;
-        const long long g = ((1ll << 15) - static_cast<long long>(sum[r]) * static_cast<long long>(f)) >> 9;
-        bt.G[r] = static_cast<uint32_t>(g);
-    }
+    for (int r = 0; r < NB; ++r)
+        row_factors_of<C>(__shfl_sync(0xffffffffu, f_own, r), sum[r], bt.F[r], bt.G[r]);
 }
 
 // Pass B of one batch: normalise and requantise the rows from registers;
@@ -211,7 +237,7 @@ __device__ __forceinline__ void pass_b(const NormParams &prm, const uint4 *cst, 
           for (int k = 0; k < 4; ++k) {
             const int ee = 3 - k;
             const int e = 4 * i + ee;
-            const uint4 rec = cst[(j * 16 + e) * 32 + lane];
+            const uint4 rec = cst[record(j, lane, e)];
             const long long b = static_cast<long long>((static_cast<unsigned long long>(rec.y) << 32) | rec.x);
 #pragma unroll
             for (int r = 0; r < NB; ++r) {
@@ -288,7 +314,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     layernorm_i8_kernel(const NormParams prm) {
     constexpr int D = 512 * C;
     extern __shared__ uint8_t smem_raw[];
-    uint4 *cst = reinterpret_cast<uint4 *>(smem_raw);   // [C * 16][32] records
+    uint4 *cst = reinterpret_cast<uint4 *>(smem_raw);
     const int lane = threadIdx.x & 31;
     // Batches are dealt warp-major (warp w of CTA c takes batch w G + c, then
     // that plus 8 G, ...), so that with fewer batches than warps every CTA,
@@ -307,39 +333,126 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
 
     // per-channel records {B' lo, B' hi, M, E - 31} with B' = B + 2^(E-1)
-    // (the rounding term folded in): channel j 512 + l 16 + e of lane l goes
-    // to record (j 16 + e) 32 + l.  When every E is at least 32 the records
-    // hold E - 32 and pass B shifts the high word of M n + B'.
+    // (the rounding term folded in): channel j 512 + l 16 + e is lane l's.  When
+    // every E is at least 32 the records
+    // hold E - 32 and pass B shifts the high word of M n + B'.  All loads go out
+    // before the first is used (in a rolled loop they waited for one another:
+    // 1 us of set-up for every 512 channels).
+    constexpr int PER = 2 * C;   // D / THREADS
+    static_assert(PER * THREADS == D, "channels per thread");
+    long long b[PER];
+    int m[PER], ex[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int k = threadIdx.x + i * THREADS;
+        b[i] = __ldg(prm.B + k);
+        m[i] = __ldg(prm.M + k);
+        ex[i] = __ldg(prm.E + k);
+    }
     bool bad = false, hi = true;
-    for (int k = threadIdx.x; k < D; k += THREADS) {
-        const int j = k >> 9, l = (k >> 4) & 31, e = k & 15;
-        long long b = prm.B[k];
-        int m = prm.M[k], ex = prm.E[k];
-        if (ex < 31 || ex > 62 || b >= (1ll << 60) || b <= -(1ll << 60)) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        if (ex[i] < 31 || ex[i] > 62 || b[i] >= (1ll << 60) || b[i] <= -(1ll << 60)) {
             bad = true;
-            ex = ex < 31 ? 31 : (ex > 62 ? 62 : ex);
-            b = 0;
+            ex[i] = ex[i] < 31 ? 31 : (ex[i] > 62 ? 62 : ex[i]);
+            b[i] = 0;
         }
-        b += 1ll << (ex - 1);
-        hi = hi && ex >= 32;
-        cst[(j * 16 + e) * 32 + l] =
-            make_uint4(static_cast<uint32_t>(b), static_cast<uint32_t>(static_cast<unsigned long long>(b) >> 32),
-                       static_cast<uint32_t>(m), static_cast<uint32_t>(ex - 31));
+        b[i] += 1ll << (ex[i] - 1);
+        hi = hi && ex[i] >= 32;
     }
     if (bad) atomicOr(prm.err, ERR_PARAM);
     const bool all_hi = __syncthreads_and(hi) != 0;
-    if (all_hi) {
-        for (int k = threadIdx.x; k < D; k += THREADS) {
-            const int j = k >> 9, l = (k >> 4) & 31, e = k & 15;
-            cst[(j * 16 + e) * 32 + l].w -= 1u;
-        }
-        __syncthreads();
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int k = threadIdx.x + i * THREADS;
+        const int j = k >> 9, l = (k >> 4) & 31, e = k & 15;
+        cst[record(j, l, e)] =
+            make_uint4(static_cast<uint32_t>(b[i]), static_cast<uint32_t>(static_cast<unsigned long long>(b[i]) >> 32),
+                       static_cast<uint32_t>(m[i]), static_cast<uint32_t>(ex[i] - (all_hi ? 32 : 31)));
     }
+    __syncthreads();
     if (!first) return;
     if (all_hi)
         run_batches<C, true>(prm, cst, grp, warps, groups, lane, bt);
     else
         run_batches<C, false>(prm, cst, grp, warps, groups, lane, bt);
+}
+
+// ---- one row per CTA ---------------------------------------------------------
+// Few rows: a warp per four rows leaves most of the GPU idle, and every CTA
+// first builds all d channel records for the few rows it has.  Here a CTA of
+// four warps takes one row: thread t the 32-bit words t + 128 k (k < C) and the
+// constants of those channels, loaded straight into registers beside the row;
+// one exchange through shared memory gives every thread the row's sums.  The
+// arithmetic is that of the batched kernel.
+constexpr int ROW_THREADS = 128;
+
+template <int C>
+__global__ void __launch_bounds__(ROW_THREADS) layernorm_row_kernel(const NormParams prm) {
+    constexpr int D = 512 * C;
+    __shared__ int part[ROW_THREADS / 32][2];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const long long row = blockIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();   // the grid before this one on the stream: complete, memory visible
+    uint32_t w[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k)
+        w[k] = __ldcs(reinterpret_cast<const uint32_t *>(prm.x + row * D) + tid + ROW_THREADS * k);
+    int m[C][4], ex[C][4];
+    long long b[C][4];
+#pragma unroll
+    for (int k = 0; k < C; ++k)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int c = 4 * (tid + ROW_THREADS * k) + e;
+            m[k][e] = __ldg(prm.M + c);
+            b[k][e] = __ldg(prm.B + c);
+            ex[k][e] = __ldg(prm.E + c);
+        }
+    int sum = 0, sq = 0;
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        sum = __dp4a(static_cast<int>(w[k]), 0x01010101, sum);
+        sq = __dp4a(static_cast<int>(w[k]), static_cast<int>(w[k]), sq);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    }
+    if (lane == 0) {
+        part[tid >> 5][0] = sum;
+        part[tid >> 5][1] = sq;
+    }
+    __syncthreads();
+    sum = part[0][0] + part[1][0] + part[2][0] + part[3][0];
+    sq = part[0][1] + part[1][1] + part[2][1] + part[3][1];
+    uint32_t F, G;
+    row_factors<C>(prm.eps_c, sum, sq, F, G);
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        int y[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            long long bb = b[k][e];
+            int x = ex[k][e];
+            if (x < 31 || x > 62 || bb >= (1ll << 60) || bb <= -(1ll << 60)) {
+                bad = true;
+                x = x < 31 ? 31 : (x > 62 ? 62 : x);
+                bb = 0;
+            }
+            const int n = static_cast<int>(static_cast<uint32_t>(sbyte(w[k], e)) * F + G) >> 7;   // |n| < 2^23
+            const long long v = static_cast<long long>(m[k][e]) * n + (bb + (1ll << (x - 1)));    // |v| < 2^62
+            const int h = static_cast<int>(__funnelshift_r(static_cast<uint32_t>(v),
+                                                           static_cast<uint32_t>(v >> 32), 31));
+            y[e] = max(h >> (x - 31), -127);
+        }
+        __stcs(reinterpret_cast<uint32_t *>(prm.y + row * D) + tid + ROW_THREADS * k,
+               pack_sat4(y[0], y[1], y[2], y[3]));
+    }
+    if (bad) atomicOr(prm.err, ERR_PARAM);
 }
 
 }  // namespace ipn
