@@ -145,6 +145,9 @@ __global__ void __launch_bounds__(DW_THREADS) dwconv_swish_kernel(const DwParams
 // products: for n = [v < 0], A = |v| and h = 2^(e-1),
 //   floor((m v + h) / 2^e) = (1 - 2n) floor((m A + h - n) / 2^e),
 // because floor((h - X) / 2h) = -floor((X + h - 1) / 2h).
+// What bounds it: integer issue, about 38 instructions per output (12000 x 1024,
+// K = 9: 25.3 us with both quotients taken at bit 31, 21.9 us at word boundaries,
+// where the high word of a product needs no shift across words).
 constexpr int DW4_THREADS = 64;      // 256 channels per CTA
 constexpr int DW4_BLOCKS = 2;        // blocks of four output frames per step
 
@@ -155,31 +158,45 @@ struct Swish16K {
 };
 
 // Eq. 7 onto the INT16 grid, then the Swish of that INT16 value onto int8
-// (Eqs. 12-13), for one channel: acc the convolution sum with bias, m and s
-// the channel's multiplier and shift, h = 2^(30+s).  The INT16 value is z =
-// (1 - 2n) a with a = min(floor((m |acc| + h - n) / 2^(31+s)), 32767); its
-// Swish product z t is (1 - 2n) U with U = a t' < 2^47, t' = 2 q_one - D^2
-// for z > 0 and D^2 for z < 0 (D = q_c - min(a, q_c)); m_sw U (up to 78 bits)
-// is split at bit 31, U = u_hi 2^31 + u_lo.  Returns the int8 in the low byte.
-__device__ __forceinline__ uint32_t dw_out(int acc, uint32_t m, int s, unsigned long long h,
+// (Eqs. 12-13), for one channel: acc the convolution sum with bias, m2 and s
+// twice the channel's multiplier and its shift, h2 = 2^(31+s).  The INT16 value
+// is z = (1 - 2n) a with a = min(floor((2 m |acc| + 2 h - 2 n) / 2^(32+s)), 32767)
+// (the numerator is below 2^64, so its high word shifted by s).  The Swish
+// product z t is (1 - 2n) U with U = a t' < 2^47, t' = 2 q_one - D^2 for z > 0
+// and D^2 for z < 0 (D = q_c - min(a, q_c)), and m_sw U has up to 78 bits.
+// WIDE_SHIFT (s_sw >= 17, the usual constants): U is split into its two words,
+// floor((m_sw U + h_sw - n) / 2^32) = m_sw u_hi + floor((m_sw u_lo + h_sw - n) /
+// 2^32) < 2^48, whose shift by s_sw - 1 fits 32 bits.  Otherwise U is split at
+// bit 31 and the quotient by 2^31 may need both words.  Returns the int8 in
+// the low byte.
+template <bool WIDE_SHIFT>
+__device__ __forceinline__ uint32_t dw_out(int acc, uint32_t m2, int s, unsigned long long h2,
                                            const Swish16K &sw) {
     const uint32_t n = acc < 0 ? 1u : 0u;
     const uint32_t A = acc < 0 ? 0u - static_cast<uint32_t>(acc) : static_cast<uint32_t>(acc);
-    const unsigned long long w = static_cast<unsigned long long>(m) * A + (h - n);   // < 2^63
-    const uint32_t R = __funnelshift_r(static_cast<uint32_t>(w), static_cast<uint32_t>(w >> 32), 31) >> s;
-    const uint32_t a = min(R, 32767u);
+    const unsigned long long w = static_cast<unsigned long long>(m2) * A + (n ? h2 - 2 : h2);
+    const uint32_t a = min(static_cast<uint32_t>(w >> 32) >> s, 32767u);
     const uint32_t dc = sw.q_c - min(a, sw.q_c);
     const uint32_t d2 = dc * dc;                          // <= q_c^2 <= q_one < 2^31
     const uint32_t tt = n ? d2 : sw.two_qone - d2;
     const unsigned long long U = static_cast<unsigned long long>(a) * tt;
-    const uint32_t ulo = static_cast<uint32_t>(U) & 0x7fffffffu;
-    const uint32_t uhi = __funnelshift_r(static_cast<uint32_t>(U), static_cast<uint32_t>(U >> 32), 31);
-    const unsigned long long w2 = static_cast<unsigned long long>(sw.m) * ulo + (sw.h - n);
-    const uint32_t f = __funnelshift_r(static_cast<uint32_t>(w2), static_cast<uint32_t>(w2 >> 32), 31);
-    const unsigned long long X = static_cast<unsigned long long>(sw.m) * uhi + f;   // < 2^48
-    const uint32_t xlo = __funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s);
-    const uint32_t xhi = static_cast<uint32_t>(X >> 32) >> sw.s;
-    const uint32_t r = xhi != 0u ? 127u : min(xlo, 127u);
+    const unsigned long long h = n ? sw.h - 1 : sw.h;
+    uint32_t r;
+    if (WIDE_SHIFT) {
+        const unsigned long long t = static_cast<unsigned long long>(sw.m) * static_cast<uint32_t>(U) + h;
+        const unsigned long long X = static_cast<unsigned long long>(sw.m) * static_cast<uint32_t>(U >> 32) +
+                                     static_cast<uint32_t>(t >> 32);
+        r = min(__funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s - 1), 127u);
+    } else {
+        const uint32_t ulo = static_cast<uint32_t>(U) & 0x7fffffffu;
+        const uint32_t uhi = __funnelshift_r(static_cast<uint32_t>(U), static_cast<uint32_t>(U >> 32), 31);
+        const unsigned long long w2 = static_cast<unsigned long long>(sw.m) * ulo + h;
+        const uint32_t f = __funnelshift_r(static_cast<uint32_t>(w2), static_cast<uint32_t>(w2 >> 32), 31);
+        const unsigned long long X = static_cast<unsigned long long>(sw.m) * uhi + f;   // < 2^48
+        const uint32_t xlo = __funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s);
+        const uint32_t xhi = static_cast<uint32_t>(X >> 32) >> sw.s;
+        r = xhi != 0u ? 127u : min(xlo, 127u);
+    }
     return n ? 0u - r : r;
 }
 
@@ -204,7 +221,7 @@ __device__ __forceinline__ void dw_transpose4(uint32_t x0, uint32_t x1, uint32_t
 // shifted by i bytes.  A step makes DW4_BLOCKS blocks of four outputs; the
 // frame words of the next step's new blocks are loaded before this step's
 // arithmetic, so their latency hides behind it.
-template <int K>
+template <int K, bool WIDE_SHIFT>
 __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *xb, uint32_t *yb,
                                             int cw, int ts, int te, const uint32_t (&wq)[4][(K + 3) / 4],
                                             const uint32_t (&mq)[4], const int (&sq)[4],
@@ -254,7 +271,7 @@ __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *x
                             i == 0 ? A[b + q][j] : __funnelshift_r(A[b + q][j], A[b + q + 1][j], 8 * i);
                         acc = __dp4a(static_cast<int>(win), static_cast<int>(wq[j][q]), acc);
                     }
-                    o[i][j] = dw_out(acc, mq[j], sq[j], hq[j], sw);
+                    o[i][j] = dw_out<WIDE_SHIFT>(acc, mq[j], sq[j], hq[j], sw);
                 }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -320,10 +337,10 @@ __global__ void __launch_bounds__(DW4_THREADS) dwconv_swish_x4_kernel(const DwPa
             ss = ss < 0 ? 0 : (ss > 31 ? 31 : ss);
             bias = 0;
         }
-        mq[j] = static_cast<uint32_t>(mm);
+        mq[j] = 2u * static_cast<uint32_t>(mm);
         sq[j] = ss;
         bq[j] = bias;
-        hq[j] = 1ull << (30 + ss);
+        hq[j] = 1ull << (31 + ss);
     }
     Swish16K sw;
     sw.q_c = static_cast<uint32_t>(p.sw_qc);
@@ -339,8 +356,12 @@ __global__ void __launch_bounds__(DW4_THREADS) dwconv_swish_x4_kernel(const DwPa
         const int ts = static_cast<int>(f - b * static_cast<uint32_t>(p.T));
         const int te = min(p.T, ts + static_cast<int>(fend - f));
         const size_t base = static_cast<size_t>(b) * p.T * cw + c4;
-        dw4_segment<K>(p, reinterpret_cast<const uint32_t *>(p.x) + base,
-                       reinterpret_cast<uint32_t *>(p.y) + base, cw, ts, te, wq, mq, sq, bq, hq, sw);
+        const uint32_t *xb = reinterpret_cast<const uint32_t *>(p.x) + base;
+        uint32_t *yb = reinterpret_cast<uint32_t *>(p.y) + base;
+        if (sw.s >= 17)
+            dw4_segment<K, true>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
+        else
+            dw4_segment<K, false>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
         f += static_cast<uint32_t>(te - ts);
     }
 }
