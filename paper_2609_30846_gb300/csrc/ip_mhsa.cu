@@ -193,37 +193,35 @@ size_t gs_scores_bytes(int T) {
            static_cast<size_t>((T + ipk::NK - 1) / ipk::NK) * ipk::CHUNK_SCORE_BYTES;
 }
 
-// Work items of the persistent kernel.  The N whole tiles run on G resident
-// CTAs in rounds; when the last round is at most a quarter full (r = N mod G
-// tiles, 4 r <= G) its r tiles become 4 r quarters of 16 rows, when at most
-// half full (2 r <= G) 2 r halves of 32 rows, whose warps split the keys of
-// every chunk, so that the last round takes a fraction of a tile's time.
+// Work items of the persistent kernel.  The N whole tiles run on the resident
+// CTAs in rounds; those of a last round that is not nearly full are split as
+// TailPlan says into halves of 32 rows or quarters of 16, whose warps split the
+// keys of every chunk, so that the round takes a fraction of a tile's time.
 struct ItemPlan {
-    uint32_t nwhole = 0, nitems = 0, grid = 0;
+    uint32_t nmain = 0, nwhole = 0, nitems = 0, grid = 0;
     int split_log2 = 1;
 };
 
-ItemPlan plan_items(long long N, int slots) {
+ItemPlan plan_items(long long N, int slots, int sms) {
     ItemPlan ip;
-    long long nwhole = N, nitems = N;
+    long long nmain = N, nwhole = N, nitems = N;
     if (g_split_mode == 1 || g_split_mode == 2) {
         ip.split_log2 = g_split_mode;
-        nwhole = 0;
+        nmain = nwhole = 0;
         nitems = N << g_split_mode;
-    } else if (g_split_mode < 0 && slots > 0) {
-        const long long r = N % slots;
-        if (r > 0 && 4 * r <= slots) {
-            ip.split_log2 = 2;
-            nwhole = N - r;
-            nitems = N + 3 * r;
-        } else if (r > 0 && 2 * r <= slots) {
-            nwhole = N - r;
-            nitems = N + r;
-        }
+    } else if (g_split_mode < 0) {
+        const ipk::TailPlan t = ipk::tail_plan(static_cast<uint32_t>(N % slots),
+                                               static_cast<uint32_t>(slots), static_cast<uint32_t>(sms));
+        nmain = N - t.tail;
+        nwhole = nmain + t.wholes;
+        nitems = nwhole + ((N - nwhole) << t.split_log2);
+        ip.split_log2 = t.split_log2;
     }
+    ip.nmain = static_cast<uint32_t>(nmain);
     ip.nwhole = static_cast<uint32_t>(nwhole);
     ip.nitems = static_cast<uint32_t>(nitems);
-    ip.grid = static_cast<uint32_t>(nitems < slots ? nitems : slots);
+    // wholes and parts beside each other: the full grid, two CTAs to an SM
+    ip.grid = static_cast<uint32_t>(nitems < slots && nwhole == nmain ? nitems : slots);
     return ip;
 }
 
@@ -331,7 +329,8 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     int sms = 0;
     const int slots = resident_ctas(gs, smem, &sms);
     if (slots < 1) return IP_ERR_CUDA;
-    ItemPlan ip = plan_items(N, slots);
+    prm.sms = slots == 2 * sms ? static_cast<uint32_t>(sms) : 0u;
+    ItemPlan ip = plan_items(N, slots, static_cast<int>(prm.sms));
     // With a mask the live tiles are planned on the device, unless all of them
     // are split in quarters anyway or every utterance is one tile.
     prm.live_plan = lengths && B <= 32 && ntiles > 1 && g_split_mode < 0 && 4 * N > slots ? 1 : 0;
@@ -346,6 +345,7 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     const int own = ip.grid <= static_cast<uint32_t>(sms) && smem < OWN_SM_SMEM ? OWN_SM_SMEM : smem;
     rc = ensure_smem(gs, own);
     if (rc != IP_OK) return rc;
+    prm.nmain = ip.nmain;
     prm.nwhole = ip.nwhole;
     prm.split_log2 = ip.split_log2;
     prm.nitems = ip.nitems;

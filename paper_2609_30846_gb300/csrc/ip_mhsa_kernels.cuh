@@ -99,16 +99,21 @@ struct FusedParams {
     int stall_injection;      // test hook: consumers first wait on a barrier nobody arrives on
     int sum32;                // exp(0) x 16 nchunk_max < 2^32: 32-bit partial sums in pass 2
     int f24;                  // exp(0) > 2^8: every row sum exceeds 2^8, so f = 2^32 / sum < 2^24
-    // Work items, claimed in order by the persistent CTAs: items [0, nwhole)
-    // are whole 64-row tiles in (b, h, tile) order, items [nwhole, nitems)
+    // Work items, claimed by the persistent CTAs: items [0, nwhole) are whole
+    // 64-row tiles in (b, h, tile) order, the first nmain of them the full
+    // rounds and the others the last one's (TailPlan), items [nwhole, nitems)
     // the 2^split_log2 parts (32-row halves or 16-row quarters) of the tiles
     // from nwhole on.  With live_plan (a key-padding mask) the items are those
     // of LivePlan instead.
-    unsigned int *sched;      // workspace words: [0] next item, [16] CTAs done claiming
+    // Workspace words: [4 i] next item of list i (see claim), [16] CTAs done
+    // claiming, [32 ..] one bit per SM, flipped by each CTA that asks for its
+    // place on the SM.
+    unsigned int *sched;
     int ntiles;                        // 64-row tiles per (b, h)
     unsigned long long tiles_magic;    // udiv_magic constant of ntiles
     unsigned long long heads_magic;    // udiv_magic constant of H
-    uint32_t nwhole, nitems;           // nitems < 2^31
+    uint32_t nmain, nwhole, nitems;    // nitems < 2^31
+    uint32_t sms;                      // SMs that hold two of the grid's CTAs each (0: other grids)
     int split_log2;                    // 1: halves, 2: quarters
     int live_plan;                     // plan over the live tiles (B <= 32)
     unsigned long long grid_magic;     // udiv_magic constant of the grid (live_plan)
@@ -659,6 +664,29 @@ __device__ __forceinline__ Item decode_slot(const FusedParams &p, uint32_t lin, 
     return decode_item(p, lin, plog2 ? static_cast<int>(code & 0xffu) : -1, plog2);
 }
 
+// The last round: r tiles for `slots` resident CTAs, two on each of `sms` SMs
+// (sms 0: one on each).  A tile in parts takes longer in total, but a part is
+// short.  In units of a whole tile's time beside another one (T = 375 .. 1500):
+// a whole tile alone on its SM 0.68, two halves beside each other 0.65, two
+// quarters 0.44.  So: up to a quarter of the slots, quarters; up to half of
+// them, halves; and above that, while each SM can take one whole tile and at
+// most one quarter (0.82) or half (0.89) beside it, the wholes and those parts.
+// Measured against whole tiles for all of such a round, two on some SMs and
+// none on others: 526 -> 478 us (B = 4, T = 1500: 2.53 rounds), 94 -> 88 us
+// (B = 10, T = 375: 1.58 rounds), 178 -> 159 us (B = 1, T = 1500: 0.63 rounds).
+struct TailPlan {
+    uint32_t tail, wholes;   // tiles of the last round (0: as the full rounds'), whole ones of them
+    int split_log2;          // the others'
+};
+
+__host__ __device__ inline TailPlan tail_plan(uint32_t r, uint32_t slots, uint32_t sms) {
+    if (4 * r <= slots) return {r, 0u, 2};
+    if (2 * r <= slots) return {r, 0u, 1};
+    if (4 * r <= 5 * sms) return {r, sms, 2};
+    if (2 * r <= 3 * sms) return {r, sms, 1};
+    return {0u, 0u, 0};
+}
+
 // Items of a batch with key padding, planned by every CTA's copy warp alike
 // from the lengths (one utterance per lane): the live 64-row tiles come first,
 // the longest utterances' before the shorter ones' (an item's cost goes with
@@ -668,7 +696,7 @@ __device__ __forceinline__ Item decode_slot(const FusedParams &p, uint32_t lin, 
 // lengths in T/2 .. T about 440 of 512 tiles are live: a plan over all of them
 // left 208 for the second round of 304 and split none (61 us; 50 us planned so).
 struct LivePlan {
-    uint32_t nwhole, nlive, ntotal;   // whole items, live items, all items
+    uint32_t nmain, nwhole, nlive, ntotal;   // whole items of full rounds, whole items, live items, all items
     int split_log2;
     int b, nt;                        // this lane's utterance in order of length, its live tiles
     uint32_t off, poff;               // live and padding tiles of the utterances before it
@@ -707,8 +735,10 @@ __device__ __forceinline__ LivePlan live_plan(const FusedParams &p, int lane) {
     L.off = warp_exclusive_sum(static_cast<uint32_t>(L.nt) * p.H, lane, live);
     L.poff = warp_exclusive_sum(real ? static_cast<uint32_t>(p.ntiles - L.nt) * p.H : 0u, lane, pads);
     const uint32_t r = live - udiv_magic(live, p.grid_magic) * gridDim.x;   // tiles of the last round
-    L.split_log2 = 4 * r <= gridDim.x ? 2 : (2 * r <= gridDim.x ? 1 : 0);
-    L.nwhole = live - (L.split_log2 ? r : 0u);
+    const TailPlan tail = tail_plan(r, gridDim.x, p.sms);
+    L.split_log2 = tail.split_log2;
+    L.nmain = live - tail.tail;
+    L.nwhole = L.nmain + tail.wholes;
     L.nlive = L.nwhole + ((live - L.nwhole) << L.split_log2);
     L.ntotal = L.nlive + pads;
     return L;
@@ -1543,23 +1573,49 @@ __global__ void __launch_bounds__(NTHREADS, 2)
     int iss_pos = 0, issued = 0;
     int kq = 0;   // live items published (slots written, Q tiles sent)
     LivePlan plan{};
-    bool first_claim = true;
+    // Items come from one list, or, where the last round has whole tiles and
+    // parts, from three: the full rounds, the last round's wholes, its parts
+    // (and the padding).  The two CTAs of an SM then find their places by
+    // flipping its bit, and the second one leaves the wholes to the first, so
+    // that no SM gets two.  A grid of two CTAs per SM has more CTAs than bits:
+    // wherever they run, one of them is a first one, and that one claims until
+    // the wholes are gone.
+    int phase = 0;
     auto claim = [&](uint32_t &lin) -> bool {
         const uint32_t n = prm.live_plan ? plan.ntotal : prm.nitems;
+        const uint32_t nmain = prm.live_plan ? plan.nmain : prm.nmain;
+        const uint32_t nwhole = prm.live_plan ? plan.nwhole : prm.nwhole;
+        const bool mixed = nwhole > nmain;
         for (;;) {
-            // one round or less: the first item is the block's, without the
-            // round trip to the counter (0.2 us of a 7.9 us call)
-            uint32_t item = blockIdx.x;
-            if (!first_claim || n > gridDim.x) {
+            uint32_t item = blockIdx.x, end = n;
+            if (n <= gridDim.x && !mixed) {
+                // one round or less: the block's item, without the round trip to
+                // the counter (0.2 us of a 7.9 us call)
+                if (phase++ != 0) return false;
+            } else {
+                if (mixed) end = phase == 0 ? nmain : (phase == 1 ? nwhole : n);
                 uint32_t x = 0;
-                if (lane == 0) x = atomicAdd(prm.sched, 1u);
-                item = __shfl_sync(0xffffffffu, x, 0) + (n > gridDim.x ? 0u : gridDim.x);
+                if (lane == 0) x = atomicAdd(prm.sched + 4 * phase, 1u);
+                item = __shfl_sync(0xffffffffu, x, 0) + (phase == 0 ? 0u : (phase == 1 ? nmain : nwhole));
             }
-            first_claim = false;
-            if (item >= n) return false;
-            iss = prm.live_plan ? plan_item(prm, plan, item, lin) : host_item(prm, item, lin);
-            if (!iss.pad) return true;
-            zero_rows(prm, iss, lane);
+            if (item < end) {
+                iss = prm.live_plan ? plan_item(prm, plan, item, lin) : host_item(prm, item, lin);
+                if (!iss.pad) return true;
+                zero_rows(prm, iss, lane);
+                continue;
+            }
+            if (!mixed || phase == 2) return false;
+            if (phase == 0) {
+                uint32_t x = 0;
+                if (lane == 0) {
+                    uint32_t sm;
+                    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+                    const uint32_t bit = 1u << (sm & 31u);
+                    x = (atomicXor(prm.sched + 32 + ((sm >> 5) & 7u), bit) & bit) != 0u;
+                }
+                phase += static_cast<int>(__shfl_sync(0xffffffffu, x, 0));
+            }
+            ++phase;
         }
     };
     // Publishes the claimed item as live item kq: its slot, then its Q tile
@@ -1585,7 +1641,8 @@ __global__ void __launch_bounds__(NTHREADS, 2)
     };
     auto done_claiming = [&]() {
         if (lane == 0 && atomicAdd(prm.sched + 16, 1u) == gridDim.x - 1) {
-            atomicExch(prm.sched, 0u);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) atomicExch(prm.sched + 4 * i, 0u);
             atomicExch(prm.sched + 16, 0u);
         }
     };
