@@ -202,8 +202,8 @@ __device__ __forceinline__ uint32_t exp_index4(uint32_t w, uint32_t mx4h) {
 }
 
 __device__ __forceinline__ uint32_t max4h(int mx0, int mx1) {
-    const uint32_t a = static_cast<uint32_t>(mx0 + 128) & 0xffu;
-    const uint32_t b = static_cast<uint32_t>(mx1 + 128) & 0xffu;
+    const uint32_t a = static_cast<uint32_t>(min(mx0, 127) + 128);
+    const uint32_t b = static_cast<uint32_t>(min(mx1, 127) + 128);
     return a | (a << 8) | (b << 16) | (b << 24);
 }
 
@@ -349,14 +349,16 @@ __device__ __forceinline__ void content_mma(int (&acc)[8][4], const uint32_t (&q
 
 // Eq. 11 for one n8 tile of the content accumulator: the fused int8 scores
 // of rows g, g+8 and keys 8nt + 2t, 8nt + 2t + 1 (Phi as the index remap
-// jj - rho + 15 into the band), key mask, running row maxima; returns the
+// jj - rho + 15 into the band), key mask, running row maxima (the clamp at 127
+// is the pack's and, of the maxima, max4h's: 238.7 -> 237.1 us at B = 32, T = 375
+// with the probabilities' clamp in their pack); returns the
 // four scores packed [g:2t, g:2t+1, g+8:2t, g+8:2t+1].
 template <bool MASK>
 __device__ __forceinline__ uint32_t score_tile(const int (&c)[4], int nt, uint32_t remap, int lane,
                                                long long m_c, long long m_p, long long half_s,
                                                int s_s, int kvalid, int &mx0, int &mx1) {
     const int g = lane >> 2, t4 = lane & 3;
-    uint32_t v[4];
+    int v[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const int rho = g + ((e >> 1) << 3);
@@ -366,13 +368,12 @@ __device__ __forceinline__ uint32_t score_tile(const int (&c)[4], int nt, uint32
         const long long x = m_c * c[e] + m_p * qp + half_s;
         const int y = static_cast<int>(__funnelshift_r(static_cast<uint32_t>(x),
                                                        static_cast<uint32_t>(x >> 32), 31));
-        int sc = min(max(y >> s_s, -127), 127);
-        if (MASK && jj >= kvalid) sc = -128;
-        if (e < 2) mx0 = max(mx0, sc);
-        else mx1 = max(mx1, sc);
-        v[e] = static_cast<uint32_t>(sc);
+        v[e] = max(y >> s_s, -127);
+        if (MASK && jj >= kvalid) v[e] = -128;
     }
-    return pack4(v[0], v[1], v[2], v[3]);
+    mx0 = __vimax3_s32(mx0, v[0], v[1]);
+    mx1 = __vimax3_s32(mx1, v[2], v[3]);
+    return pack_sat4(v[0], v[1], v[2], v[3]);
 }
 
 // Eq. 11 for a whole chunk (8 tiles) and the store of the packed scores.
@@ -437,7 +438,7 @@ template <bool B> struct BoolTag {
 // grid 2^-8: min(floor(ev f / 2^24), 255).  Masked keys (score -128) are
 // zeroed by the caller.  F24: every row sum exceeds 2^8, so f < 2^24 and
 // the callers pass f0, f1 times 2^8: the floor is then the high word of
-// ev (f 2^8).  Otherwise, with ev f = hi 2^32 + lo, it is 255 when hi > 0,
+// ev (f 2^8), at most 2^8 since ev is a term of the sum.  Otherwise, with ev f = hi 2^32 + lo, it is 255 when hi > 0,
 // else lo >> 24 (at most 255).
 template <bool F24>
 __device__ __forceinline__ uint32_t prob_word(uint32_t wv, uint32_t lut_g, uint32_t mx4h,
@@ -449,11 +450,11 @@ __device__ __forceinline__ uint32_t prob_word(uint32_t wv, uint32_t lut_g, uint3
         const uint32_t f = e < 2 ? f0 : f1;
         const uint32_t ev = lds32(lut_at(lut_g, d4, e));
         if (F24)
-            a[e] = min(__umulhi(ev, f), 255u);
+            a[e] = __umulhi(ev, f);
         else
             a[e] = __umulhi(ev, f) != 0u ? 255u : (ev * f) >> 24;
     }
-    return pack4(a[0], a[1], a[2], a[3]);
+    return F24 ? pack_satu4(a[0], a[1], a[2], a[3]) : pack4(a[0], a[1], a[2], a[3]);
 }
 
 // Byte mask of a probability word of tile q of a 32-key step whose first

@@ -255,6 +255,14 @@ __device__ __forceinline__ uint32_t pack_sat4(int y0, int y1, int y2, int y3) {
     return pack_sat2(y1, y0, pack_sat2(y3, y2, 0u));
 }
 
+// Bytes [y0, y1, y2, y3] of four values below 2^31, each saturated to [0, 255].
+__device__ __forceinline__ uint32_t pack_satu4(uint32_t y0, uint32_t y1, uint32_t y2, uint32_t y3) {
+    uint32_t hi, w;
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(y3), "r"(y2));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(y1), "r"(y0), "r"(hi));
+    return w;
+}
+
 // Sign-extended byte e (0..3) of w: one prmt, byte e in the low byte and
 // its sign bit replicated in the three above (selector bit 3).
 __device__ __forceinline__ int sbyte(uint32_t w, int e) {
