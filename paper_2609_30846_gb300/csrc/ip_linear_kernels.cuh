@@ -163,13 +163,15 @@ constexpr int EPI_RES = 3;     // requantised int8, then the residual addition t
 
 // Eq. 7 for one accumulator (with its bias): max(round(m acc / 2^(31 + s)), -127)
 // with rnd = 2^(30 + s); the callers clamp at 127 (a saturating pack).
-// |m acc| < 2^62, so the quotient by 2^31 is a 32-bit value (funnel
-// shift) and the rest is a shift by s.
-__device__ __forceinline__ int requant(int acc, int cm, int cs, long long rnd) {
+// |m acc| < 2^62, so the quotient by 2^31 is a 32-bit value (funnel shift) and
+// the rest is a shift by s.  HI (s >= 1): the high word and a shift by sh = s - 1.
+template <bool HI>
+__device__ __forceinline__ int requant(int acc, int cm, int sh, long long rnd) {
     const long long v = static_cast<long long>(cm) * acc + rnd;
-    const int h = static_cast<int>(__funnelshift_r(static_cast<uint32_t>(v),
-                                                   static_cast<uint32_t>(v >> 32), 31));
-    return max(h >> cs, -127);
+    const int h = HI ? static_cast<int>(v >> 32)
+                     : static_cast<int>(__funnelshift_r(static_cast<uint32_t>(v),
+                                                        static_cast<uint32_t>(v >> 32), 31));
+    return max(h >> sh, -127);
 }
 
 // One stage of a dp4a unit: lane (rg, cg) of RG row and CG channel groups
@@ -246,6 +248,10 @@ __device__ __forceinline__ uint32_t atom_inc(uint32_t addr, uint32_t limit) {
     asm volatile("atom.acq_rel.cta.shared.inc.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(limit) : "memory");
     return old;
 }
+
+template <int V> struct IntConst {
+    static constexpr int value = V;
+};
 
 // Word of tile element (row, col) in a group's partial sums: the channel
 // index XORed with the row, so that the fragment stores of an MMA warp (four
@@ -463,44 +469,66 @@ __global__ void __launch_bounds__(THREADS, 2)
 #pragma unroll
         for (int e = 0; e < 4; ++e) rnd[e] = 1ll << (30 + cs[e]);
     }
-#pragma unroll
-    for (int q = 0; q < C::ROUNDS; ++q) {
-        if (flat0 + STEP * q >= frames) break;
-        int a[4] = {cb[0], cb[1], cb[2], cb[3]};
-#pragma unroll
-        for (int g = 0; g < C::NG; ++g) {
-            const uint4 v = lds128(ring + g * (C::OUT * 4) + part_at<TN>(rl + STEP * q, cl));
-            a[0] += static_cast<int>(v.x);
-            a[1] += static_cast<int>(v.y);
-            a[2] += static_cast<int>(v.z);
-            a[3] += static_cast<int>(v.w);
-        }
-        int z[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) z[e] = requant(a[e], cm[e], cs[e], rnd[e]);
+    // One loop per epilogue, shift form and layout, chosen once per tile: the
+    // epilogue's instructions take issue slots from the other CTA's dp4a warps
+    // (of 331 us at 1024 -> 3072, 12000 frames, 20 us went with it; 324 us with
+    // the choices out of the loop and the shift below).  HI: every channel of the
+    // warp has s >= 1, and the quotient by 2^(31 + s) is the high word >> (s - 1).
+    auto rows = [&](auto epi_tag, auto hi_tag, auto heads_tag) {
+        constexpr int EPI = decltype(epi_tag)::value;
+        constexpr bool HI = decltype(hi_tag)::value != 0, HEADS = decltype(heads_tag)::value != 0;
         int8_t *dst = prm.y + off;
-        if (glu) {
-            // channels (a_c, b_c) interleaved: two gated outputs
-            const uint32_t w = (static_cast<uint32_t>(glu_i8(min(z[0], 127), min(z[1], 127), prm)) & 0xffu) |
-                               ((static_cast<uint32_t>(glu_i8(min(z[2], 127), min(z[3], 127), prm)) & 0xffu) << 8);
-            *reinterpret_cast<uint16_t *>(dst) = static_cast<uint16_t>(w);
-        } else {
-            uint32_t w = pack_sat4(z[0], z[1], z[2], z[3]);
-            if (prm.epi == EPI_SWISH)
-                w = swish_lut[w & 0xffu] | (swish_lut[(w >> 8) & 0xffu] << 8) |
-                    (swish_lut[(w >> 16) & 0xffu] << 16) | (static_cast<uint32_t>(swish_lut[w >> 24]) << 24);
-            else if (prm.epi == EPI_RES)
-                w = residual4(xr[q], w, prm.res_mx, prm.res_my, prm.res_s);
-            *reinterpret_cast<uint32_t *>(dst) = w;
+        int sh[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sh[e] = HI ? cs[e] - 1 : cs[e];
+#pragma unroll
+        for (int q = 0; q < C::ROUNDS; ++q) {
+            if (flat0 + STEP * q >= frames) break;
+            int a[4] = {cb[0], cb[1], cb[2], cb[3]};
+#pragma unroll
+            for (int g = 0; g < C::NG; ++g) {
+                const uint4 v = lds128(ring + g * (C::OUT * 4) + part_at<TN>(rl + STEP * q, cl));
+                a[0] += static_cast<int>(v.x);
+                a[1] += static_cast<int>(v.y);
+                a[2] += static_cast<int>(v.z);
+                a[3] += static_cast<int>(v.w);
+            }
+            int z[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) z[e] = requant<HI>(a[e], cm[e], sh[e], rnd[e]);
+            if (EPI == EPI_GLU) {
+                // channels (a_c, b_c) interleaved: two gated outputs
+                const uint32_t w = (static_cast<uint32_t>(glu_i8(min(z[0], 127), min(z[1], 127), prm)) & 0xffu) |
+                                   ((static_cast<uint32_t>(glu_i8(min(z[2], 127), min(z[3], 127), prm)) & 0xffu) << 8);
+                *reinterpret_cast<uint16_t *>(dst) = static_cast<uint16_t>(w);
+            } else {
+                uint32_t w = pack_sat4(z[0], z[1], z[2], z[3]);
+                if (EPI == EPI_SWISH)
+                    w = swish_lut[w & 0xffu] | (swish_lut[(w >> 8) & 0xffu] << 8) |
+                        (swish_lut[(w >> 16) & 0xffu] << 16) | (static_cast<uint32_t>(swish_lut[w >> 24]) << 24);
+                else if (EPI == EPI_RES)
+                    w = residual4(xr[q], w, prm.res_mx, prm.res_my, prm.res_s);
+                *reinterpret_cast<uint32_t *>(dst) = w;
+            }
+            if (HEADS) {
+                dst += STEP << 7;
+                for (t += STEP; t >= prm.T; t -= prm.T)   // into the next utterance
+                    dst += static_cast<long long>(prm.heads_per_group - 1) * prm.T << 7;
+            } else {
+                dst += STEP * width;
+            }
         }
-        if (heads) {
-            off += STEP << 7;
-            for (t += STEP; t >= prm.T; t -= prm.T)   // into the next utterance
-                off += static_cast<long long>(prm.heads_per_group - 1) * prm.T << 7;
-        } else {
-            off += STEP * width;
-        }
-    }
+    };
+    const bool hi = __all_sync(0xffffffffu, cs[0] > 0 && cs[1] > 0 && cs[2] > 0 && cs[3] > 0) != 0;
+    auto by_shift = [&](auto epi_tag, auto heads_tag) {
+        if (hi) rows(epi_tag, IntConst<1>(), heads_tag);
+        else rows(epi_tag, IntConst<0>(), heads_tag);
+    };
+    if (heads) by_shift(IntConst<EPI_PLAIN>(), IntConst<1>());
+    else if (prm.epi == EPI_PLAIN) by_shift(IntConst<EPI_PLAIN>(), IntConst<0>());
+    else if (prm.epi == EPI_SWISH) by_shift(IntConst<EPI_SWISH>(), IntConst<0>());
+    else if (prm.epi == EPI_GLU) by_shift(IntConst<EPI_GLU>(), IntConst<0>());
+    else by_shift(IntConst<EPI_RES>(), IntConst<0>());
 }
 
 }  // namespace ipl
