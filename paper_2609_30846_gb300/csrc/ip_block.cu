@@ -62,7 +62,7 @@ cudaError_t launch_dw4(ipb::DwParams p, cudaStream_t st) {
     long long per_block = slots / ncb > 0 ? slots / ncb : 1;
     // a multiple of the frames of one step, so that only utterance ends
     // leave a partly used step
-    constexpr int step = 4 * ipb::DW4_BLOCKS;
+    constexpr int step = 4;
     const long long per = ((frames + per_block - 1) / per_block + step - 1) / step * step;
     per_block = (frames + per - 1) / per;
     p.frames_per_cta = static_cast<uint32_t>(per);
@@ -139,6 +139,11 @@ int ip_dwconv_swish_i8(const int8_t *x, int B, int T, int C, const int8_t *w, in
     p.K = K;
     p.sw_qc = sw->q_c;
     p.sw_qone = sw->q_one;
+    // the most negative Swish product is that of z = -q_c / 3: -4 q_c^3 / 27
+    const __int128 c3 = static_cast<__int128>(sw->q_c) * sw->q_c * sw->q_c;
+    p.sw_fast = sw->s >= 17 && sw->q_c <= 32767 && sw->q_one < (1 << 30) &&
+                        sw->m * (4 * c3 / 27 + 1) <= (static_cast<__int128>(127) << (31 + sw->s))
+                    ? 1 : 0;
     p.sw_m = sw->m;
     p.sw_s = sw->s;
     p.err = static_cast<int *>(workspace);

@@ -56,6 +56,7 @@ struct DwParams {
     int B, T, C, K;
     int sw_qc, sw_m, sw_s;    // Swish of the INT16 value onto int8
     long long sw_qone;
+    int sw_fast;              // the constants fit dw_out's 32-bit form
     int *err;
     // four-channels-per-thread kernel: CTA (j, cb) takes channel block cb
     // and the frames [j per, (j + 1) per) of the B T frames in (b, t) order
@@ -140,64 +141,59 @@ __global__ void __launch_bounds__(DW_THREADS) dwconv_swish_kernel(const DwParams
 // consecutive frames of one channel each), so that one dp4a covers four
 // taps: output frame t of channel c is the sum over q of dp4a(the four
 // frames t - K/2 + 4q .. + 3, taps 4q .. 4q + 3), the frame words taken at
-// any byte offset by a funnel shift of two neighbouring channel words.  The
-// two roundings are done in sign and magnitude with 32 x 32 -> 64-bit
-// products: for n = [v < 0], A = |v| and h = 2^(e-1),
-//   floor((m v + h) / 2^e) = (1 - 2n) floor((m A + h - n) / 2^e),
-// because floor((h - X) / 2h) = -floor((X + h - 1) / 2h).
-// What bounds it: integer issue, about 38 instructions per output (12000 x 1024,
-// K = 9: 25.3 us with both quotients taken at bit 31, 21.9 us at word boundaries,
-// where the high word of a product needs no shift across words).
+// any byte offset by a funnel shift of two neighbouring channel words.
+// What bounds it: instruction issue, and most of all the pipe of the integer
+// multiplies (every multiply, dp4a, shift, permute and pack takes two cycles of a
+// pipe per warp, additions and minima one).  So the two quotients are taken at word
+// boundaries on signed products, a thread makes four frames at a time (eight kept
+// more registers and fewer warps: 21.6 us), and ten CTAs of 64 threads share an SM
+// (96 registers; with eight, 128 registers, the largest case is 2 % faster, but 1332
+// frames take 6.3 us).  12000 x 1024, K = 9: 25.3 -> 21.0 us; K = 15: 27.7 -> 22.6;
+// 12000 x 512, K = 5: 17.0 -> 11.0; 1332 x 1024, K = 9: 7.6 -> 5.3; 125 x 1024: 2.8 -> 2.2.
 constexpr int DW4_THREADS = 64;      // 256 channels per CTA
-constexpr int DW4_BLOCKS = 2;        // blocks of four output frames per step
 
 struct Swish16K {
-    uint32_t q_c, two_qone, m;
+    int q_c;
+    uint32_t two_qone, m;
     int s;
     unsigned long long h;            // 2^(30+s)
 };
 
 // Eq. 7 onto the INT16 grid, then the Swish of that INT16 value onto int8
-// (Eqs. 12-13), for one channel: acc the convolution sum with bias, m2 and s
-// twice the channel's multiplier and its shift, h2 = 2^(31+s).  The INT16 value
-// is z = (1 - 2n) a with a = min(floor((2 m |acc| + 2 h - 2 n) / 2^(32+s)), 32767)
-// (the numerator is below 2^64, so its high word shifted by s).  The Swish
-// product z t is (1 - 2n) U with U = a t' < 2^47, t' = 2 q_one - D^2 for z > 0
-// and D^2 for z < 0 (D = q_c - min(a, q_c)), and m_sw U has up to 78 bits.
-// WIDE_SHIFT (s_sw >= 17, the usual constants): U is split into its two words,
-// floor((m_sw U + h_sw - n) / 2^32) = m_sw u_hi + floor((m_sw u_lo + h_sw - n) /
-// 2^32) < 2^48, whose shift by s_sw - 1 fits 32 bits.  Otherwise U is split at
-// bit 31 and the quotient by 2^31 may need both words.  Returns the int8 in
-// the low byte.
-template <bool WIDE_SHIFT>
-__device__ __forceinline__ uint32_t dw_out(int acc, uint32_t m2, int s, unsigned long long h2,
-                                           const Swish16K &sw) {
-    const uint32_t n = acc < 0 ? 1u : 0u;
-    const uint32_t A = acc < 0 ? 0u - static_cast<uint32_t>(acc) : static_cast<uint32_t>(acc);
-    const unsigned long long w = static_cast<unsigned long long>(m2) * A + (n ? h2 - 2 : h2);
-    const uint32_t a = min(static_cast<uint32_t>(w >> 32) >> s, 32767u);
-    const uint32_t dc = sw.q_c - min(a, sw.q_c);
-    const uint32_t d2 = dc * dc;                          // <= q_c^2 <= q_one < 2^31
-    const uint32_t tt = n ? d2 : sw.two_qone - d2;
-    const unsigned long long U = static_cast<unsigned long long>(a) * tt;
-    const unsigned long long h = n ? sw.h - 1 : sw.h;
-    uint32_t r;
-    if (WIDE_SHIFT) {
-        const unsigned long long t = static_cast<unsigned long long>(sw.m) * static_cast<uint32_t>(U) + h;
-        const unsigned long long X = static_cast<unsigned long long>(sw.m) * static_cast<uint32_t>(U >> 32) +
-                                     static_cast<uint32_t>(t >> 32);
-        r = min(__funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s - 1), 127u);
+// (Eqs. 12-13), for one channel: acc the convolution sum with bias, m the
+// channel's multiplier, h2 = 2^(31 + s).  z = clamp(floor((m 2 acc + h2) / 2^(32 + s)))
+// and the Swish product is U = z t, |U| < 2^47, with t = 2 q_one - D^2 for z > 0,
+// D^2 for z < 0 (D = max(q_c - |z|, 0)).  m_sw U has up to 78 bits: with U = u_hi
+// 2^32 + u_lo (u_hi signed, u_lo not), its floor by 2^32 is X = m_sw u_hi +
+// floor((m_sw u_lo + h_sw) / 2^32), |X| < 2^48, and signs need no case of their own.
+// FAST, the usual constants (the host's DwParams::sw_fast, and |bias| of the
+// thread's channels at most DW_BIAS, so that 2 acc is a 32-bit value and the first
+// quotient a high word shifted by s): t fits a signed word, X shifted by s_sw - 1
+// fits 32 bits; z < -32767 needs no clamp, since D = 0 from -q_c on; and no negative
+// output is below -127.  Otherwise quotients and clamps are taken in 64 bits.  The
+// clamp of the output at 127 is the pack's.
+constexpr int DW_BIAS = (1 << 30) - (1 << 20);   // + 127 127 K < 2^30
+
+template <bool FAST>
+__device__ __forceinline__ int dw_out(int acc, int m, int s, long long h2, const Swish16K &sw) {
+    int z;
+    if (FAST) {
+        const long long w = static_cast<long long>(m) * (2 * acc) + h2;   // < 2^62 + 2^62
+        z = min(static_cast<int>(w >> 32) >> s, 32767);
     } else {
-        const uint32_t ulo = static_cast<uint32_t>(U) & 0x7fffffffu;
-        const uint32_t uhi = __funnelshift_r(static_cast<uint32_t>(U), static_cast<uint32_t>(U >> 32), 31);
-        const unsigned long long w2 = static_cast<unsigned long long>(sw.m) * ulo + h;
-        const uint32_t f = __funnelshift_r(static_cast<uint32_t>(w2), static_cast<uint32_t>(w2 >> 32), 31);
-        const unsigned long long X = static_cast<unsigned long long>(sw.m) * uhi + f;   // < 2^48
-        const uint32_t xlo = __funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s);
-        const uint32_t xhi = static_cast<uint32_t>(X >> 32) >> sw.s;
-        r = xhi != 0u ? 127u : min(xlo, 127u);
+        const long long w = static_cast<long long>(m) * acc + (h2 >> 1);
+        z = static_cast<int>(max(min(w >> (31 + s), 32767ll), -32767ll));
     }
-    return n ? 0u - r : r;
+    const int dc = max(sw.q_c - abs(z), 0);
+    const int d2 = dc * dc;                               // <= q_c^2 <= q_one < 2^31
+    const uint32_t tt = z > 0 ? sw.two_qone - static_cast<uint32_t>(d2) : static_cast<uint32_t>(d2);
+    const long long U = FAST ? static_cast<long long>(z) * static_cast<int>(tt) : static_cast<long long>(z) * static_cast<long long>(tt);
+    const unsigned long long t = static_cast<unsigned long long>(sw.m) * static_cast<uint32_t>(U) + sw.h;
+    const long long X = static_cast<long long>(sw.m) * static_cast<int>(U >> 32) + static_cast<uint32_t>(t >> 32);
+    if (FAST) return static_cast<int>(__funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s - 1));
+    // the quotient by 2^31 of the whole needs bit 31 of t too where s_sw = 0
+    const long long Y = sw.s > 0 ? X >> (sw.s - 1) : 2 * X + static_cast<long long>((t >> 31) & 1u);
+    return static_cast<int>(max(min(Y, 127ll), -127ll));
 }
 
 // Byte transpose of a 4x4 block: y_c = [x0.b_c, x1.b_c, x2.b_c, x3.b_c].
@@ -218,18 +214,16 @@ __device__ __forceinline__ void dw_transpose4(uint32_t x0, uint32_t x1, uint32_t
 // [0, T) read as zero): block u holds frames p0 + 4u .. p0 + 4u + 3, as one
 // channel word per channel.  Output frame ts + 4v + i reads the stream at
 // offsets 4v + i .. 4v + i + K - 1, i.e. the words of blocks v .. v + Q
-// shifted by i bytes.  A step makes DW4_BLOCKS blocks of four outputs; the
-// frame words of the next step's new blocks are loaded before this step's
-// arithmetic, so their latency hides behind it.
-template <int K, bool WIDE_SHIFT>
+// shifted by i bytes.  A step makes one block of four outputs; the frame words
+// of the next step's new block are loaded before this step's arithmetic, so
+// their latency hides behind it.
+template <int K, bool FAST>
 __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *xb, uint32_t *yb,
                                             int cw, int ts, int te, const uint32_t (&wq)[4][(K + 3) / 4],
-                                            const uint32_t (&mq)[4], const int (&sq)[4],
-                                            const int (&bq)[4], const unsigned long long (&hq)[4],
+                                            const int (&mq)[4], const int (&sq)[4],
+                                            const int (&bq)[4], const long long (&hq)[4],
                                             const Swish16K &sw) {
     constexpr int Q = (K + 3) / 4;    // weight words (taps in fours)
-    constexpr int NB = DW4_BLOCKS;
-    constexpr int NA = Q + NB;        // blocks a step reads
     const int T = p.T;
     const int p0 = ts - (K >> 1);
     auto load_block = [&](int u, uint32_t (&xw)[4]) {
@@ -239,52 +233,41 @@ __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *x
             xw[r] = (tt >= 0 && tt < T) ? __ldg(xb + static_cast<size_t>(tt) * cw) : 0u;
         }
     };
-    uint32_t A[NA][4];   // A[u][j]: channel j of block NB v + u for step v
-    uint32_t nx[NB][4];  // frame words of the next step's new blocks
+    uint32_t A[Q + 1][4];   // A[u][j]: channel j of block v + u for step v
+    uint32_t nx[4];         // frame words of the next step's new block
 #pragma unroll
     for (int u = 0; u < Q; ++u) {
-        load_block(u, nx[0]);
-        dw_transpose4(nx[0][0], nx[0][1], nx[0][2], nx[0][3], A[u]);
+        load_block(u, nx);
+        dw_transpose4(nx[0], nx[1], nx[2], nx[3], A[u]);
     }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) load_block(Q + b, nx[b]);
-    const int nsteps = (te - ts + 4 * NB - 1) / (4 * NB);
+    load_block(Q, nx);
+    const int nsteps = (te - ts + 3) / 4;
 #pragma unroll 1
     for (int v = 0; v < nsteps; ++v) {
+        dw_transpose4(nx[0], nx[1], nx[2], nx[3], A[Q]);
+        if (v + 1 < nsteps) load_block(v + 1 + Q, nx);
+        int o[4][4];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) dw_transpose4(nx[b][0], nx[b][1], nx[b][2], nx[b][3], A[Q + b]);
-        if (v + 1 < nsteps) {
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int b = 0; b < NB; ++b) load_block(NB * (v + 1) + Q + b, nx[b]);
-        }
+            for (int j = 0; j < 4; ++j) {
+                int acc = bq[j];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-            uint32_t o[4][4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    int acc = bq[j];
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) {
-                        const uint32_t win =
-                            i == 0 ? A[b + q][j] : __funnelshift_r(A[b + q][j], A[b + q + 1][j], 8 * i);
-                        acc = __dp4a(static_cast<int>(win), static_cast<int>(wq[j][q]), acc);
-                    }
-                    o[i][j] = dw_out<WIDE_SHIFT>(acc, mq[j], sq[j], hq[j], sw);
+                for (int q = 0; q < Q; ++q) {
+                    const uint32_t win = i == 0 ? A[q][j] : __funnelshift_r(A[q][j], A[q + 1][j], 8 * i);
+                    acc = __dp4a(static_cast<int>(win), static_cast<int>(wq[j][q]), acc);
                 }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int t = ts + 4 * (NB * v + b) + i;
-                if (t < te)
-                    yb[static_cast<size_t>(t) * cw] = __byte_perm(
-                        __byte_perm(o[i][0], o[i][1], 0x0040), __byte_perm(o[i][2], o[i][3], 0x0040), 0x5410);
+                o[i][j] = dw_out<FAST>(acc, mq[j], sq[j], hq[j], sw);
             }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = ts + 4 * v + i;
+            if (t < te) yb[static_cast<size_t>(t) * cw] = pack_sat4(o[i][0], o[i][1], o[i][2], o[i][3]);
         }
 #pragma unroll
         for (int u = 0; u < Q; ++u)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) A[u][j] = A[u + NB][j];
+            for (int j = 0; j < 4; ++j) A[u][j] = A[u + 1][j];
     }
 }
 
@@ -293,7 +276,7 @@ __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *x
 // split at utterance boundaries (the zero padding of each utterance).  The
 // grid holds one CTA per resident slot, so there is no partial second wave.
 template <int K>
-__global__ void __launch_bounds__(DW4_THREADS) dwconv_swish_x4_kernel(const DwParams p) {
+__global__ void __launch_bounds__(DW4_THREADS, 10) dwconv_swish_x4_kernel(const DwParams p) {
     pdl_launch_dependents();
     pdl_wait();   // the grid before this one on the stream: complete, memory visible
     constexpr int Q = (K + 3) / 4;
@@ -324,9 +307,9 @@ __global__ void __launch_bounds__(DW4_THREADS) dwconv_swish_x4_kernel(const DwPa
                 wq[j][q] = v;
             }
     }
-    uint32_t mq[4];
-    int sq[4], bq[4];
-    unsigned long long hq[4];
+    int mq[4], sq[4], bq[4];
+    long long hq[4];
+    bool fast = p.sw_fast != 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int c = 4 * c4 + j;
@@ -337,13 +320,14 @@ __global__ void __launch_bounds__(DW4_THREADS) dwconv_swish_x4_kernel(const DwPa
             ss = ss < 0 ? 0 : (ss > 31 ? 31 : ss);
             bias = 0;
         }
-        mq[j] = 2u * static_cast<uint32_t>(mm);
+        mq[j] = mm;
         sq[j] = ss;
         bq[j] = bias;
-        hq[j] = 1ull << (31 + ss);
+        hq[j] = 1ll << (31 + ss);
+        fast &= bias <= DW_BIAS && bias >= -DW_BIAS;
     }
     Swish16K sw;
-    sw.q_c = static_cast<uint32_t>(p.sw_qc);
+    sw.q_c = p.sw_qc;
     sw.two_qone = static_cast<uint32_t>(2 * p.sw_qone);
     sw.m = static_cast<uint32_t>(p.sw_m);
     sw.s = p.sw_s;
@@ -358,7 +342,7 @@ __global__ void __launch_bounds__(DW4_THREADS) dwconv_swish_x4_kernel(const DwPa
         const size_t base = static_cast<size_t>(b) * p.T * cw + c4;
         const uint32_t *xb = reinterpret_cast<const uint32_t *>(p.x) + base;
         uint32_t *yb = reinterpret_cast<uint32_t *>(p.y) + base;
-        if (sw.s >= 17)
+        if (fast)
             dw4_segment<K, true>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
         else
             dw4_segment<K, false>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
