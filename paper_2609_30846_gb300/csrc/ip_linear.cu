@@ -73,9 +73,9 @@ using LinearKernel = void (*)(const CUtensorMap, const CUtensorMap, const ipl::L
 // so a wave of one tile per SM takes half of what a pair does).  Fitted on
 // GB300 to sweeps of M = 16 .. 12000 frames over N = 512 .. 4096 and K = 1024 ..
 // 4096 (all four shapes timed at each point; the model is at most 11 % off, and
-// its choice at most 5 % slower than the best of the four, 0.3 % on average).  A large tile costs the least per output, a small one fills the SMs:
-// at K = 1024, N = 4096 one 64 x 128 tile per SM takes 15.9 us, 32 x 32 tiles
-// 4.1 us at M = 30, and at M = 12000 451 us against 667 us.
+// its choice at most 5 % slower than the best of the four, 0.3 % on average).  A
+// large tile costs the least per output, a small one fills the SMs: at K = 1024, N = 4096 one 64 x 128 tile per SM takes 15.9 us, 32 x 32 tiles
+// 4.1 us at M = 30, and at M = 12000 435 us against 667 us.
 struct Variant {
     LinearKernel fn;
     int tm, tn;

@@ -25,9 +25,9 @@
 // frames of all utterances form one axis of B T rows; with a head-split X a
 // tile stays inside one utterance.
 //
-// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 9.1 us, 12000 frames
-// 460 -> 451 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 9.3 us,
-// 1332 frames 87.9 -> 57.8 us, 12000 frames 431 -> 410 us (before: one
+// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 8.6 us, 12000 frames
+// 460 -> 435 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 9.2 us,
+// 1332 frames 87.9 -> 59.1 us, 12000 frames 431 -> 409 us (before: one
 // persistent CTA of 17 warps per SM over 128 x 128 tiles, the channels of a
 // tile split between the pipes: a short batch filled 8 to 32 of the SMs, and
 // every lane computed the address of each of its shared loads).

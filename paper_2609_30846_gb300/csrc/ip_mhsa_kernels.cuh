@@ -11,14 +11,14 @@
 //
 // The CTAs are persistent (one per resident slot) and take work items in
 // turn: a whole 64-row tile of one (b, h), or, for the tail of the work, a
-// 32-row half of one.  Four consumer warps of 16 rows and two producer
-// warps: the copy warp issues the TMA loads through a two-stage ring that
+// 32-row half or a 16-row quarter of one.  Four consumer warps of 16 rows and
+// two producer warps: the copy warp issues the TMA loads through a two-stage ring that
 // runs on across items (the next item's first chunks are in flight while
 // the current one finishes), and the bias warp computes the bias vectors
 // K u and P v of each staged score-pass chunk (the exact rank-1 split of
 // (Q + 1u^T)K^T and (Q + 1v^T)P^T, since Q + u does not fit an int8
-// operand).  The attn.V pass reads the V tile as TMA stages it: transposed
-// ldmatrix loads and byte selects build the MMA operand.
+// operand).  The attn.V pass reads the V tile as TMA stages it: 8-bit
+// transposing ldmatrix loads give the MMA operand.
 // The consumers, per item:
 //   pass 1  for each chunk of 64 keys: the content MMAs Q K^T, the MMAs of
 //           the position band Q P_band^T for the next chunk (issued before
@@ -49,7 +49,7 @@ constexpr int NK = 64;                    // keys per chunk
 constexpr int NSTAGE = 2;
 constexpr int BAND_ROWS = 128;            // P rows staged per chunk (NK + MROWS - 1, padded)
 constexpr int K_TILE_BYTES = NK * DH;     // K (pass 1) or V (pass 3) tile
-constexpr int P_TILE_BYTES = BAND_ROWS * DH;   // P band (pass 1) or transposed V (pass 3)
+constexpr int P_TILE_BYTES = BAND_ROWS * DH;   // P band (pass 1)
 constexpr int KU_OFF = K_TILE_BYTES + P_TILE_BYTES;   // int32 K u of the chunk's keys
 constexpr int PV_OFF = KU_OFF + NK * 4;                // int32 P v of the band rows
 constexpr int STAGE_BYTES = 25600;        // PV_OFF + BAND_ROWS * 4, rounded to 1024
@@ -568,7 +568,7 @@ __device__ __forceinline__ void send_partial(const int (&oacc)[16][4], uint32_t 
 
 // Adds the partner's partial sums of this warp's n-tiles 8 HK .. 8 HK + 7
 // (d = 64 HK .. 64 HK + 63), requantises them (Eq. 7) and stores four bytes
-// per row and d chunk: d = 16c + 4t .. 16c + 4t + 3 for c in 4 HK .. 4 HK + 3.
+// per row and d chunk c in 4 HK .. 4 HK + 3 (out_words).
 template <int HK>
 __device__ __forceinline__ void finish_half(int (&oacc)[16][4], uint32_t pxo, int lane, int wrow0,
                                             int len, const FusedParams &prm, int b, int h) {
@@ -1055,7 +1055,7 @@ __device__ __forceinline__ bool consume_whole(const FusedParams &prm, const Item
     if (!ok3) return false;
 
     // ---- output requantisation (Eq. 7): per d chunk c and row, four bytes
-    // d = 16c + 4t .. 16c + 4t + 3 (n-tiles 2c, 2c + 1, columns 2t, 2t + 1).
+    // 16c + out_col .. + 3 (n-tiles 2c, 2c + 1).
     // The d chunks go in the order their last MMAs were issued, so the
     // first ones are requantised while the pipe finishes the others.
     int8_t *const dst0 = prm.out + out_offset(prm, it.b, it.h, wrow0 + g) + out_col(t4);
