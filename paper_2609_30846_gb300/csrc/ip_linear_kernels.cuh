@@ -25,9 +25,9 @@
 // frames of all utterances form one axis of B T rows; with a head-split X a
 // tile stays inside one utterance.
 //
-// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 8.6 us, 12000 frames
-// 460 -> 435 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 9.2 us,
-// 1332 frames 87.9 -> 59.1 us, 12000 frames 431 -> 409 us (before: one
+// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 8.4 us, 12000 frames
+// 460 -> 432 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 9.1 us,
+// 1332 frames 87.9 -> 58.2 us, 12000 frames 431 -> 408 us (before: one
 // persistent CTA of 17 warps per SM over 128 x 128 tiles, the channels of a
 // tile split between the pipes: a short batch filled 8 to 32 of the SMs, and
 // every lane computed the address of each of its shared loads).
@@ -77,6 +77,7 @@ struct Shape {
     static constexpr int RING = (NEXT + 4 + 1023) & ~1023;
     // shared memory of a CTA with pg stages per group (+ alignment of the base)
     static constexpr int smem(int pg) { return RING + pg * NG * STAGE + 1024; }
+    static constexpr int AREAS = NG >> 1;         // areas of partial sums: one per pair of groups
     static_assert(WPG <= 4 && NG >= 2, "groups");
     static_assert((STAGE & 1023) == 0 && (A_BYTES & 1023) == 0, "128-byte swizzle");
 };
@@ -249,6 +250,11 @@ __device__ __forceinline__ uint32_t atom_inc(uint32_t addr, uint32_t limit) {
     return old;
 }
 
+// Adds v to a word of shared memory.
+__device__ __forceinline__ void red_add(uint32_t addr, int v) {
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
 template <int V> struct IntConst {
     static constexpr int value = V;
 };
@@ -370,8 +376,11 @@ __global__ void __launch_bounds__(THREADS, 2)
         }
     };
 
-    // Partial sums of the group, written over the ring once every warp has
-    // read its last stage.
+    // Partial sums of the groups, written over the ring once every warp has read
+    // its last stage: the MMA groups store theirs and the dp4a groups add to them
+    // (one group each), so that the epilogue reads half as many words.  With an
+    // area per group: 324.4 -> 321.7 us (12000 x 1024 -> 3072), 59.1 -> 58.2 (1332 x
+    // 4096 -> 1024), 8.67 -> 8.44 (125 x 1024 -> 4096).
     auto all_done = [&]() -> bool {
         if (__syncthreads_or(ok ? 0 : 1) == 0) return true;
         if (threadIdx.x == 0)   // let the copies in flight land before the CTA exits
@@ -379,7 +388,7 @@ __global__ void __launch_bounds__(THREADS, 2)
                 if (issued[s] >= 0) mbar_wait(full_bar(s), issued[s] & 1, 2000000000ll);
         return false;
     };
-    const uint32_t part = ring + grp * (C::OUT * 4);
+    const uint32_t part = ring + gi * (C::OUT * 4);
     if (on_mma) {
         constexpr int MI = C::MU_M >> 4, NI = C::MU_N >> 3;
         constexpr int UL = lg2(TM) - lg2(C::MU_M);   // units along the frames: 1 << UL
@@ -402,6 +411,7 @@ __global__ void __launch_bounds__(THREADS, 2)
                 for (int rr = 0; rr < 2; ++rr)
                     sts64(part + part_at<TN>(r0 + 16 * i + g + 8 * rr, c0 + 8 * j + 2 * t4),
                           acc[i][j][2 * rr], acc[i][j][2 * rr + 1]);
+        __syncthreads();
     } else {
         constexpr int CG = C::DU_N >> 3, RI = C::DU_M >> lg2(32 >> lg2(CG));
         constexpr int UL = lg2(TM) - lg2(C::DU_M);
@@ -416,12 +426,14 @@ __global__ void __launch_bounds__(THREADS, 2)
             dp4a_stage<RI, CG>(acc, st + r0 * 128, st + C::A_BYTES + c0 * 128, rg, cg);
         });
         if (!all_done()) return;
+        __syncthreads();   // the MMA warps' sums are there
 #pragma unroll
         for (int i = 0; i < RI; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                sts32(part + part_at<TN>(r0 + rg + (32 >> lg2(CG)) * i, c0 + cg + CG * j),
-                      static_cast<uint32_t>(acc[i][j]));
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t at = part + part_at<TN>(r0 + rg + (32 >> lg2(CG)) * i, c0 + cg + CG * j);
+                red_add(at, acc[i][j]);
+            }
     }
 
     // ------------------------------------------------------------ epilogue
@@ -486,7 +498,7 @@ __global__ void __launch_bounds__(THREADS, 2)
             if (flat0 + STEP * q >= frames) break;
             int a[4] = {cb[0], cb[1], cb[2], cb[3]};
 #pragma unroll
-            for (int g = 0; g < C::NG; ++g) {
+            for (int g = 0; g < C::AREAS; ++g) {
                 const uint4 v = lds128(ring + g * (C::OUT * 4) + part_at<TN>(rl + STEP * q, cl));
                 a[0] += static_cast<int>(v.x);
                 a[1] += static_cast<int>(v.y);
