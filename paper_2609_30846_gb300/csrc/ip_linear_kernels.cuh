@@ -25,9 +25,9 @@
 // frames of all utterances form one axis of B T rows; with a head-split X a
 // tile stays inside one utterance.
 //
-// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 8.4 us, 12000 frames
-// 460 -> 432 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 9.1 us,
-// 1332 frames 87.9 -> 58.2 us, 12000 frames 431 -> 408 us (before: one
+// Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 8.2 us, 12000 frames
+// 460 -> 425 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 8.7 us,
+// 1332 frames 87.9 -> 56.8 us, 12000 frames 431 -> 405 us (before: one
 // persistent CTA of 17 warps per SM over 128 x 128 tiles, the channels of a
 // tile split between the pipes: a short batch filled 8 to 32 of the SMs, and
 // every lane computed the address of each of its shared loads).
@@ -50,9 +50,9 @@ __host__ __device__ constexpr int lg2(int x) { return x <= 1 ? 0 : 1 + lg2(x >> 
 
 // Shape of one CTA's work.  A unit is what one warp accumulates: 2048
 // outputs (64 x 32 or 32 x 64; 64 per lane) or, for the smallest tile, 1024.
-// The warps whose units cover the tile once form a group; the groups take
-// the K stages in turn, so a group's accumulators are partial sums over its
-// stages, added through shared memory at the end.
+// The warps whose units cover the tile once form a group; the groups share
+// the K stages, so a group's accumulators are partial sums over its stages,
+// added through shared memory at the end.
 template <int TM_, int TN_>
 struct Shape {
     static constexpr int TM = TM_, TN = TN_;      // frames x channels
@@ -72,9 +72,8 @@ struct Shape {
     static constexpr int CONSTS = 0;              // bias, multiplier, shift of the TN channels
     static constexpr int LUT = CONSTS + 3 * 4 * TN;
     static constexpr int BARS = LUT + 256;
-    static constexpr int SLOT_INFO = BARS + 8 * MAX_SLOTS;   // per slot: uses issued, end mark, warps done
-    static constexpr int NEXT = SLOT_INFO + 12 * MAX_SLOTS;    // next stage to claim
-    static constexpr int RING = (NEXT + 4 + 1023) & ~1023;
+    static constexpr int SLOT_INFO = BARS + 8 * MAX_SLOTS;   // per slot: uses issued, warps done
+    static constexpr int RING = (SLOT_INFO + 8 * MAX_SLOTS + 1023) & ~1023;
     // shared memory of a CTA with pg stages per group (+ alignment of the base)
     static constexpr int smem(int pg) { return RING + pg * NG * STAGE + 1024; }
     static constexpr int AREAS = NG >> 1;         // areas of partial sums: one per pair of groups
@@ -282,9 +281,7 @@ __global__ void __launch_bounds__(THREADS, 2)
     const uint32_t base = smem_u32(smem), ring = base + C::RING;
     auto full_bar = [&](int s) { return base + C::BARS + 8u * s; };
     volatile int *issued = reinterpret_cast<int *>(smem + C::SLOT_INFO);
-    volatile int *ended = issued + MAX_SLOTS;
-    int *next = reinterpret_cast<int *>(smem + C::NEXT);
-    const uint32_t done = base + C::SLOT_INFO + 8 * MAX_SLOTS;   // per slot: warps done with its stage
+    const uint32_t done = base + C::SLOT_INFO + 4 * MAX_SLOTS;   // per slot: warps done with its stage
     const uint8_t *swish_lut = smem + C::LUT;
     const int slots = C::NG * prm.pg;
 
@@ -293,8 +290,6 @@ __global__ void __launch_bounds__(THREADS, 2)
         mbar_init(full_bar(threadIdx.x), 1);
         sts32(done + 4u * threadIdx.x, 0u);
         issued[threadIdx.x] = -1;
-        ended[threadIdx.x] = 0;
-        if (threadIdx.x == 0) *next = slots;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -303,22 +298,23 @@ __global__ void __launch_bounds__(THREADS, 2)
     pdl_wait();   // the grid before this one on the stream: complete, memory visible
 
     // Warps 0-3 run the integer MMA pipe, 4-7 the dp4a pipe (one of each on
-    // every SM sub-partition).  Each group has pg slots of the ring (group g:
-    // slots g, g + NG, ...) and uses them in turn; when a slot has been
-    // consumed, the group's first warp claims the next stage of K for it, so
-    // the faster pipe takes more stages.  A slot without a stage is marked
-    // ended and its barrier completed without a copy.
+    // every SM sub-partition).  The MMA groups take the first half of the stages
+    // of K in turn, the dp4a groups the second, each through its own pg slots of
+    // the ring (g, g + NG, ...); the last of a group's warps to finish a stage
+    // refills its slot.  What a warp does between two stages adds to the time in
+    // full (three more shared loads there: 5 %), so the split is fixed: with stages
+    // claimed from a counter, and an end mark to read in each slot, 321.8 us against
+    // 316.7 (12000 x 1024 -> 3072), 408.7 against 405.0 (12000 x 4096 -> 1024), 3.80
+    // against 3.60 (125 x 1024 -> 1024).  The halves are equal: at K = 4096 17 of 32
+    // stages on the MMA pipe take 412.5 us, 18 take 427.
     const bool on_mma = warp < 4;
     const int gi = C::WPG == 1 ? (warp & 3) : (C::WPG == 2 ? (warp & 3) >> 1 : 0);
     const int u = (warp & 3) & (C::WPG - 1);
     const int grp = 2 * gi + (on_mma ? 0 : 1);
+    const int mma_kt = (kt + 1) >> 1, pairs = C::NG / 2;
+    const int begin = (on_mma ? 0 : mma_kt) + gi, last = on_mma ? mma_kt : kt;
+    const int ahead = prm.pg * pairs;   // stages of the pipe between two uses of a slot
     auto issue = [&](int it, int slot, int use) {
-        if (it >= kt) {
-            ended[slot] = 1;
-            issued[slot] = -1;   // its copies have been consumed
-            mbar_arrive(full_bar(slot));
-            return;
-        }
         const uint32_t st = ring + slot * C::STAGE;
         issued[slot] = use;
         mbar_expect_tx(full_bar(slot), C::STAGE);
@@ -329,7 +325,7 @@ __global__ void __launch_bounds__(THREADS, 2)
         tma_load_2d(st + C::A_BYTES, &tm_w, it * BK, L.n0, full_bar(slot));
     };
     if (u == 0 && lane == 0)
-        for (int slot = grp; slot < slots; slot += C::NG) issue(slot, slot, 0);
+        for (int it = begin, slot = grp; slot < slots && it < last; it += pairs, slot += C::NG) issue(it, slot, 0);
 
     // while the first stages land: the channel constants (clipped into their
     // domain) and the Swish of every int8 input, entry at the byte value of z
@@ -355,19 +351,22 @@ __global__ void __launch_bounds__(THREADS, 2)
 
     bool ok = true;
     auto run_stages = [&](auto &&compute) {
-        for (int slot = grp, use = 0;;) {
+        for (int it = begin, slot = grp, use = 0; it < last; it += pairs) {
             if (!warp_wait(full_bar(slot), use & 1, prm.timeout_cycles)) {
                 if (lane == 0) atomicOr(prm.err, 1);
                 ok = false;
                 return;
             }
-            if (ended[slot]) return;
             compute(ring + slot * C::STAGE);
-            // the last warp of the group to finish refills the slot: nobody waits
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0 && (C::WPG == 1 || atom_inc(done + 4u * slot, C::WPG - 1) == C::WPG - 1))
-                issue(atomicAdd(next, 1), slot, use + 1);
+            const bool refill = it + ahead < last;
+            // Without a refill the fence can go: 1332 x 4096 -> 1024 57.0 -> 56.8 us; the
+            // largest shape runs 0.5 % faster with it always there.
+            if (refill || C::NG == 2) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0 && refill && (C::WPG == 1 || atom_inc(done + 4u * slot, C::WPG - 1) == C::WPG - 1))
+                    issue(it + ahead, slot, use + 1);
+            }
             slot += C::NG;
             if (slot >= slots) {
                 slot = grp;
