@@ -72,10 +72,13 @@ using LinearKernel = void (*)(const CUtensorMap, const CUtensorMap, const ipl::L
 // `base + w (wave + wave_k kt)` with w = ceil(n / SMs) (two CTAs share an SM,
 // so a wave of one tile per SM takes half of what a pair does).  Fitted on
 // GB300 to sweeps of M = 16 .. 12000 frames over N = 512 .. 4096 and K = 1024 ..
-// 4096 (all four shapes timed at each point; the model is at most 11 % off, and
-// its choice at most 5 % slower than the best of the four, 0.3 % on average).  A
-// large tile costs the least per output, a small one fills the SMs: at K = 1024, N = 4096 one 64 x 128 tile per SM takes 15.9 us, 32 x 32 tiles
-// 4.1 us at M = 30, and at M = 12000 435 us against 667 us.
+// 4096 with all four shapes timed at each point, and 400 added to `one`: such a
+// CTA holds all of an SM's shared memory, so that the launches before and after
+// it cannot share the SM (without it the block of one 10 s utterance takes 95.5
+// us for 90.3, and ties fall on the slower side).  The choice is at most 0.5 %
+// slower than the best of the four on the swept points.  A large tile costs the least per
+// output, a small one fills the SMs: at K = 1024, N = 4096 64 x 128 tiles take 13.9
+// us at M = 30, 32 x 32 ones 3.7 us, and at M = 12000 425 us against 624 us.
 struct Variant {
     LinearKernel fn;
     int tm, tn;
@@ -91,10 +94,10 @@ constexpr Variant variant(int one, int one_k, int base, int wave, int wave_k) {
             ipl::Shape<TM, TN>::smem(PG2), one, one_k, base, wave, wave_k};
 }
 const Variant VARIANTS[] = {
-    variant<64, 128, 4, 2>(3900, 1500, 3500, 1730, 1196),
-    variant<64, 64, 3, 1>(3100, 752, 2800, 1130, 627),
-    variant<32, 64, 2, 1>(2750, 376, 2500, 800, 313),
-    variant<32, 32, 3, 1>(2200, 224, 1900, 770, 170),
+    variant<64, 128, 4, 2>(3241, 1445, 2816, 816, 1259),
+    variant<64, 64, 3, 1>(2768, 741, 2246, 655, 647),
+    variant<32, 64, 2, 1>(2800, 371, 2353, 547, 321),
+    variant<32, 32, 3, 1>(2422, 207, 1681, 542, 171),
 };
 
 int ensure_smem() {

@@ -13,10 +13,11 @@ pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-# (B, T, K): with N = 2048 the host picks 32 x 32 tiles up to 64 frames, then
-# 32 x 64, 64 x 64 (from 129) and 64 x 128 (from 289 at K = 128, 1505 at K = 1152)
+# (B, T, K): with N = 2048 the host picks 32 x 32 tiles for up to 128 frames at
+# K = 128, 64 x 64 from 129, 32 x 64 from 257 and 64 x 128 from 289; 32 x 64 from 225
+# and 64 x 128 from 1505 at K = 1152
 SIZES = [(1, 1, 128), (2, 32, 1152), (5, 13, 128), (1, 127, 384), (3, 43, 128), (1, 256, 384), (17, 17, 128),
-         (2, 192, 128), (8, 190, 1152)]
+         (2, 192, 128), (8, 190, 1152), (1, 257, 128), (2, 200, 384), (15, 17, 1152)]
 
 
 @pytest.fixture(scope="module")
