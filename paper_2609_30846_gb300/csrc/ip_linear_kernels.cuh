@@ -27,7 +27,7 @@
 //
 // Measured (1024 -> 4096 with Swish): 125 frames 24.9 -> 8.2 us, 12000 frames
 // 460 -> 425 us; 4096 -> 1024 with the residual: 125 frames 87.6 -> 8.7 us,
-// 1332 frames 87.9 -> 56.8 us, 12000 frames 431 -> 405 us (before: one
+// 1332 frames 87.9 -> 55.3 us, 12000 frames 431 -> 405 us (before: one
 // persistent CTA of 17 warps per SM over 128 x 128 tiles, the channels of a
 // tile split between the pipes: a short batch filled 8 to 32 of the SMs, and
 // every lane computed the address of each of its shared loads).
