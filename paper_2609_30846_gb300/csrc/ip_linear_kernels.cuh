@@ -163,15 +163,15 @@ constexpr int EPI_RES = 3;     // requantised int8, then the residual addition t
 
 // Eq. 7 for one accumulator (with its bias): max(round(m acc / 2^(31 + s)), -127)
 // with rnd = 2^(30 + s); the callers clamp at 127 (a saturating pack).
-// |m acc| < 2^62, so the quotient by 2^31 is a 32-bit value (funnel shift) and
-// the rest is a shift by s.  HI (s >= 1): the high word and a shift by sh = s - 1.
+// |acc| < 2^30 + 2^29 (a bias below 2^30 and 32768 products of at most 2^14), so
+// |m acc| < 3 2^60, and the rounding term adds 2^(30 + s), up to 2^61: the sum stays
+// below 5 2^60, and its quotient by 2^(31 + s) is a 32-bit value for every s, but
+// the one by 2^31 alone only for s = 0.  HI (s >= 1): the high word and a shift by
+// sh = s - 1; else a 64-bit shift by sh = 31 + s.
 template <bool HI>
 __device__ __forceinline__ int requant(int acc, int cm, int sh, long long rnd) {
     const long long v = static_cast<long long>(cm) * acc + rnd;
-    const int h = HI ? static_cast<int>(v >> 32)
-                     : static_cast<int>(__funnelshift_r(static_cast<uint32_t>(v),
-                                                        static_cast<uint32_t>(v >> 32), 31));
-    return max(h >> sh, -127);
+    return max(HI ? static_cast<int>(v >> 32) >> sh : static_cast<int>(v >> sh), -127);
 }
 
 // One stage of a dp4a unit: lane (rg, cg) of RG row and CG channel groups
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(THREADS, 2)
         int8_t *dst = prm.y + off;
         int sh[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) sh[e] = HI ? cs[e] - 1 : cs[e];
+        for (int e = 0; e < 4; ++e) sh[e] = HI ? cs[e] - 1 : cs[e] + 31;
 #pragma unroll
         for (int q = 0; q < C::ROUNDS; ++q) {
             if (flat0 + STEP * q >= frames) break;
