@@ -67,37 +67,44 @@ int sm_count() {
 
 using LinearKernel = void (*)(const CUtensorMap, const CUtensorMap, const ipl::LinearParams);
 
-// The kernel's tile shapes, and what a launch of n tiles costs with each (ns,
-// kt = K / 128): with one tile per SM or less `one + one_k kt`, else
-// `base + w (wave + wave_k kt)` with w = ceil(n / SMs) (two CTAs share an SM,
-// so a wave of one tile per SM takes half of what a pair does).  Fitted on
-// GB300 to sweeps of M = 16 .. 12000 frames over N = 512 .. 4096 and K = 1024 ..
-// 4096 with all four shapes timed at each point, and 400 added to `one`: such a
+// The kernel's tile shapes, and what a launch of n tiles costs with each (ns): with
+// one tile per SM or less `one + one_r r + one_k kt`, else `base + w (wave + wave_r
+// r + wave_k kt)`, where kt = K / 128, r is kt rounded up to the shape's groups of
+// warps (they take a stage each at a time: 125 x 128 -> 1024 in 32 x 64 tiles takes as
+// long as 125 x 1024 -> 1024, 5.2 and 5.7 us), and w = ceil(n / SMs) (two CTAs share
+// an SM, so a wave of one tile per SM takes half of what a pair does).  Fitted on
+// GB300 to sweeps of M = 1 .. 12000 frames over N = 128 .. 16384 and eighteen K from
+// 128 to 8192 with all four shapes timed at each point, and 400 added to `one`: such a
 // CTA holds all of an SM's shared memory, so that the launches before and after
 // it cannot share the SM (without it the block of one 10 s utterance takes 95.5
-// us for 90.3, and ties fall on the slower side).  The choice is at most 0.5 %
-// slower than the best of the four on the swept points.  A large tile costs the least per
-// output, a small one fills the SMs: at K = 1024, N = 4096 64 x 128 tiles take 13.9
-// us at M = 30, 32 x 32 ones 3.7 us, and at M = 12000 425 us against 624 us.
+// us for 90.3, and ties fall on the slower side).  On the swept points the choice is
+// 0.1 % slower than the best of the four in the mean, 30 % at most (one frame, K = N =
+// 8192: 35 us for 27).  A large tile costs the least per output, a small one fills the
+// SMs: at K = 1024, N = 4096 64 x 128 tiles take 13.9 us at M = 30, 32 x 32 ones 3.7
+// us, and at M = 12000 425 us against 624 us.  A model without r, fitted at K = 1024
+// and more, took too small a tile where K is short or no multiple of 1024: 500 x 256 ->
+// 8192 22.5 us for 15.2, 333 x 512 -> 16384 53.5 for 35.4, 500 x 1152 -> 4096 35.4 for 27.1.
 struct Variant {
     LinearKernel fn;
     int tm, tn;
     int pg1, pg2;         // ring stages per group with one and with two CTAs on an SM
     int smem1, smem2;
-    int one, one_k, base, wave, wave_k;
+    int one, one_r, one_k, base, wave, wave_r, wave_k;
+    int groups;
 };
 template <int TM, int TN, int PG1, int PG2>
-constexpr Variant variant(int one, int one_k, int base, int wave, int wave_k) {
+constexpr Variant variant(int one, int one_r, int one_k, int base, int wave, int wave_r, int wave_k) {
     static_assert(PG1 * ipl::Shape<TM, TN>::NG <= ipl::MAX_SLOTS, "slots");
     static_assert(TM * TN * 4 <= PG2 * ipl::Shape<TM, TN>::STAGE, "the partial sums reuse the ring");
     return {ipl::linear_i8_kernel<TM, TN>, TM, TN, PG1, PG2, ipl::Shape<TM, TN>::smem(PG1),
-            ipl::Shape<TM, TN>::smem(PG2), one, one_k, base, wave, wave_k};
+            ipl::Shape<TM, TN>::smem(PG2), one, one_r, one_k, base, wave, wave_r, wave_k,
+            ipl::Shape<TM, TN>::NG};
 }
 const Variant VARIANTS[] = {
-    variant<64, 128, 4, 2>(3241, 1445, 2816, 816, 1259),
-    variant<64, 64, 3, 1>(2768, 741, 2246, 655, 647),
-    variant<32, 64, 2, 1>(2800, 371, 2353, 547, 321),
-    variant<32, 32, 3, 1>(2422, 207, 1681, 542, 171),
+    variant<64, 128, 4, 2>(3430, 1143, 309, 3117, 579, 611, 628),
+    variant<64, 64, 3, 1>(3118, 624, 120, 3042, 402, 443, 203),
+    variant<32, 64, 2, 1>(3057, 327, 49, 3129, 433, 185, 131),
+    variant<32, 32, 3, 1>(2641, 181, 32, 2289, 503, 90, 79),
 };
 
 int ensure_smem() {
@@ -130,7 +137,9 @@ const Variant &choose_variant(int x_layout, int B, int T, int K, int N, int nsm)
     for (const Variant &v : VARIANTS) {
         const long long n = tiles_of(v, x_layout, B, T, N), kt = K / ipl::BK;
         const long long w = (n + nsm - 1) / nsm;
-        const long long ns = w <= 1 ? v.one + v.one_k * kt : v.base + w * (v.wave + v.wave_k * kt);
+        const long long r = (kt + v.groups - 1) / v.groups * v.groups;
+        const long long ns = w <= 1 ? v.one + v.one_r * r + v.one_k * kt
+                                    : v.base + w * (v.wave + v.wave_r * r + v.wave_k * kt);
         if (least < 0 || ns < least) {
             least = ns;
             best = &v;

@@ -34,10 +34,10 @@ def _d(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-# with K = 1152 and N = 2048 the host picks tiles of 32 x 32, 32 x 64, 64 x 64
-# (449 to 576 frames) and 64 x 128, more than one per SM; nine stages of K, so
-# that slots of the ring are refilled
-@pytest.mark.parametrize("T", [96, 240, 500, 1601])
+# with K = 1152 and N = 2048 the host picks tiles of 32 x 32, 32 x 64 (353 to 448
+# frames), 64 x 64 (609 to 896) and 64 x 128, more than one per SM; nine stages of
+# K, so that slots of the ring are refilled
+@pytest.mark.parametrize("T", [96, 400, 700, 1601])
 def test_rounding_term_at_shift_31(ip, orc, T):
     K, N = 1152, 2048
     c = synth.linear(1, T, K, N, seed=31 + T)
