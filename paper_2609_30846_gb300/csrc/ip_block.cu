@@ -30,30 +30,31 @@ int sm_count() {
     return g_sms[dev];
 }
 
-// Resident CTAs of dwconv_swish_x4_kernel<K> on the current device (SMs x
-// CTAs per SM), looked up once per device and K.
-int g_dw4_slots[64][ipb::DW_KMAX + 1] = {{0}};
+// Resident CTAs of a dwconv_swish_x4_kernel on the current device (SMs x CTAs
+// per SM), looked up once per device and kernel.
+int g_dw4_slots[64][ipb::DW_KMAX + 1][4] = {{{0}}};
 
-template <int K>
-cudaError_t launch_dw4(ipb::DwParams p, cudaStream_t st) {
+template <int K, int FORM, int CTAS>
+cudaError_t launch_dw4_as(ipb::DwParams p, cudaStream_t st) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    constexpr int kernel = CTAS > 1 ? 3 : FORM;
     int slots = 0;
     {
         std::lock_guard<std::mutex> lock(g_mu);
-        slots = g_dw4_slots[dev][K];
+        slots = g_dw4_slots[dev][K][kernel];
     }
     if (slots == 0) {
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ipb::dwconv_swish_x4_kernel<K>,
-                                                          ipb::DW4_THREADS, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, ipb::dwconv_swish_x4_kernel<K, FORM, CTAS>, ipb::DW4_THREADS, 0);
         if (e != cudaSuccess) return e;
         slots = (per_sm > 0 ? per_sm : 1) * sm_count();
         if (slots <= 0) return cudaErrorInvalidValue;
         std::lock_guard<std::mutex> lock(g_mu);
-        g_dw4_slots[dev][K] = slots;
+        g_dw4_slots[dev][K][kernel] = slots;
     }
     // channel blocks of 256 channels; the frames of each split evenly over
     // the slots left for it
@@ -67,9 +68,25 @@ cudaError_t launch_dw4(ipb::DwParams p, cudaStream_t st) {
     per_block = (frames + per - 1) / per;
     p.frames_per_cta = static_cast<uint32_t>(per);
     p.t_magic = iph::div_magic(static_cast<unsigned long long>(p.T));
-    return iph::launch_pdl(ipb::dwconv_swish_x4_kernel<K>,
+    return iph::launch_pdl(ipb::dwconv_swish_x4_kernel<K, FORM, CTAS>,
                            dim3(static_cast<unsigned>(per_block), static_cast<unsigned>(ncb)),
                            dim3(ipb::DW4_THREADS), 0, st, p);
+}
+
+template <int K>
+cudaError_t launch_dw4(const ipb::DwParams &p, cudaStream_t st) {
+    if (p.sw_form == ipb::DW_FULL) return launch_dw4_as<K, ipb::DW_FULL, 1>(p, st);
+    if (p.sw_form == ipb::DW_WIDE) return launch_dw4_as<K, ipb::DW_WIDE, 1>(p, st);
+    return launch_dw4_as<K, ipb::DW_FAST, 10>(p, st);
+}
+
+// The form of dw_out that the constants fit.  No negative output below -127: the
+// most negative Swish product is that of z = -q_c / 3, -4 q_c^3 / 27.
+int swish16_form(const ip_swish16_params *sw) {
+    const __int128 c3 = static_cast<__int128>(sw->q_c) * sw->q_c * sw->q_c;
+    if (sw->s < 17 || sw->m * (4 * c3 / 27 + 1) > (static_cast<__int128>(127) << (31 + sw->s)))
+        return ipb::DW_FULL;
+    return sw->q_c <= 32767 && sw->q_one < (1 << 30) ? ipb::DW_FAST : ipb::DW_WIDE;
 }
 
 int check_swish16(const ip_swish16_params *p) {
@@ -139,11 +156,7 @@ int ip_dwconv_swish_i8(const int8_t *x, int B, int T, int C, const int8_t *w, in
     p.K = K;
     p.sw_qc = sw->q_c;
     p.sw_qone = sw->q_one;
-    // the most negative Swish product is that of z = -q_c / 3: -4 q_c^3 / 27
-    const __int128 c3 = static_cast<__int128>(sw->q_c) * sw->q_c * sw->q_c;
-    p.sw_fast = sw->s >= 17 && sw->q_c <= 32767 && sw->q_one < (1 << 30) &&
-                        sw->m * (4 * c3 / 27 + 1) <= (static_cast<__int128>(127) << (31 + sw->s))
-                    ? 1 : 0;
+    p.sw_form = swish16_form(sw);
     p.sw_m = sw->m;
     p.sw_s = sw->s;
     p.err = static_cast<int *>(workspace);

@@ -56,7 +56,7 @@ struct DwParams {
     int B, T, C, K;
     int sw_qc, sw_m, sw_s;    // Swish of the INT16 value onto int8
     long long sw_qone;
-    int sw_fast;              // the constants fit dw_out's 32-bit form
+    int sw_form;              // DW_FAST, DW_WIDE or DW_FULL: the form of dw_out the constants fit
     int *err;
     // four-channels-per-thread kernel: CTA (j, cb) takes channel block cb
     // and the frames [j per, (j + 1) per) of the B T frames in (b, t) order
@@ -161,39 +161,74 @@ struct Swish16K {
 
 // Eq. 7 onto the INT16 grid, then the Swish of that INT16 value onto int8
 // (Eqs. 12-13), for one channel: acc the convolution sum with bias, m the
-// channel's multiplier, h2 = 2^(31 + s).  z = clamp(floor((m 2 acc + h2) / 2^(32 + s)))
-// and the Swish product is U = z t, |U| < 2^47, with t = 2 q_one - D^2 for z > 0,
-// D^2 for z < 0 (D = max(q_c - |z|, 0)).  m_sw U has up to 78 bits: with U = u_hi
-// 2^32 + u_lo (u_hi signed, u_lo not), its floor by 2^32 is X = m_sw u_hi +
-// floor((m_sw u_lo + h_sw) / 2^32), |X| < 2^48, and signs need no case of their own.
-// FAST, the usual constants (the host's DwParams::sw_fast, and |bias| of the
-// thread's channels at most DW_BIAS, so that 2 acc is a 32-bit value and the first
-// quotient a high word shifted by s): t fits a signed word, X shifted by s_sw - 1
-// fits 32 bits; z < -32767 needs no clamp, since D = 0 from -q_c on; and no negative
-// output is below -127.  Otherwise quotients and clamps are taken in 64 bits.  The
-// clamp of the output at 127 is the pack's.
-constexpr int DW_BIAS = (1 << 30) - (1 << 20);   // + 127 127 K < 2^30
+// channel's multiplier, h2 = 2^(31 + s).  z = clamp(floor((m acc + h2 / 2) / 2^(31 +
+// s))) and the Swish product is U = z t, |U| < 2^47, with t = 2 q_one - D^2 for z > 0,
+// D^2 for z < 0 (D = max(q_c - |z|, 0)).  m_sw U has up to 78 bits.  The forms
+// differ in what fits a word; the host picks one by the Swish constants
+// (swish16_form), and the clamp of the output at 127 is the pack's.
+//
+// DW_FAST and DW_WIDE work on signed products: with U = u_hi 2^32 + u_lo (u_hi signed,
+// u_lo not), floor(m_sw U / 2^32) is X = m_sw u_hi + floor((m_sw u_lo + h_sw) / 2^32),
+// |X| < 2^46, and signs need no case of their own.  X shifted by s_sw - 1 >= 16 fits
+// a word, and no negative output is below -127.
+// DW_FAST, the usual constants (an INT16 range from 5.7 on, and |bias| of the
+// thread's channels at most DW_BIAS): 2 acc is a 32-bit value, so that the first
+// quotient is a high word shifted by s; t fits a signed word; and z < -32767 needs
+// no clamp, since D = 0 from -q_c on.
+// DW_WIDE (a range of 4.02, the least that q_one < 2^31 allows, to 5.7, or any
+// bias): a 64-bit shift gives the first quotient (a 32-bit value for every shift,
+// since |acc| < 2^30 + 2^18), z is clamped on both sides, and t is unsigned.
+// DW_FULL, any other constants of the domain, in sign and magnitude with 32 x 32 ->
+// 64-bit products: for n = [v < 0], A = |v| and h = 2^(e-1), floor((m v + h) / 2^e) =
+// (1 - 2n) floor((m A + h - n) / 2^e), because floor((h - X) / 2h) = -floor((X + h -
+// 1) / 2h); m_sw U is split at bit 31.
+// 12000 x 1024, K = 9: FAST 20.1 us, WIDE 22.8, FULL 22.7.  Quotients and clamps of
+// signed values in 64 bits for all that is not FAST took 30.2.
+constexpr int DW_FAST = 0, DW_WIDE = 1, DW_FULL = 2;
+constexpr int DW_BIAS = (1 << 30) - (1 << 20);   // + 128 128 K < 2^30
 
-template <bool FAST>
+template <int FORM>
 __device__ __forceinline__ int dw_out(int acc, int m, int s, long long h2, const Swish16K &sw) {
+    if (FORM == DW_FULL) {
+        const uint32_t n = acc < 0 ? 1u : 0u;
+        const uint32_t A = acc < 0 ? 0u - static_cast<uint32_t>(acc) : static_cast<uint32_t>(acc);
+        const unsigned long long w = static_cast<unsigned long long>(static_cast<uint32_t>(m)) * A +
+                                     (static_cast<unsigned long long>(h2 >> 1) - n);   // < 2^63
+        const uint32_t a = min(static_cast<uint32_t>(w >> (31 + s)), 32767u);
+        const uint32_t q_c = static_cast<uint32_t>(sw.q_c), dc = q_c - min(a, q_c);
+        const uint32_t d2 = dc * dc;                          // <= q_c^2 <= q_one < 2^31
+        const uint32_t tt = n ? d2 : sw.two_qone - d2;
+        const unsigned long long U = static_cast<unsigned long long>(a) * tt;
+        const uint32_t ulo = static_cast<uint32_t>(U) & 0x7fffffffu;
+        const uint32_t uhi = __funnelshift_r(static_cast<uint32_t>(U), static_cast<uint32_t>(U >> 32), 31);
+        const unsigned long long w2 = static_cast<unsigned long long>(sw.m) * ulo + (sw.h - n);
+        const uint32_t f = __funnelshift_r(static_cast<uint32_t>(w2), static_cast<uint32_t>(w2 >> 32), 31);
+        const unsigned long long X = static_cast<unsigned long long>(sw.m) * uhi + f;   // < 2^48
+        const uint32_t xlo = __funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s);
+        const uint32_t xhi = static_cast<uint32_t>(X >> 32) >> sw.s;
+        const uint32_t r = xhi != 0u ? 127u : min(xlo, 127u);
+        return static_cast<int>(n ? 0u - r : r);
+    }
     int z;
-    if (FAST) {
+    if (FORM == DW_FAST) {
         const long long w = static_cast<long long>(m) * (2 * acc) + h2;   // < 2^62 + 2^62
         z = min(static_cast<int>(w >> 32) >> s, 32767);
     } else {
         const long long w = static_cast<long long>(m) * acc + (h2 >> 1);
-        z = static_cast<int>(max(min(w >> (31 + s), 32767ll), -32767ll));
+        z = max(min(static_cast<int>(w >> (31 + s)), 32767), -32767);
     }
     const int dc = max(sw.q_c - abs(z), 0);
     const int d2 = dc * dc;                               // <= q_c^2 <= q_one < 2^31
     const uint32_t tt = z > 0 ? sw.two_qone - static_cast<uint32_t>(d2) : static_cast<uint32_t>(d2);
-    const long long U = FAST ? static_cast<long long>(z) * static_cast<int>(tt) : static_cast<long long>(z) * static_cast<long long>(tt);
+    long long U;
+    if (FORM == DW_FAST)
+        U = static_cast<long long>(z) * static_cast<int>(tt);
+    else   // the unsigned product is 2^32 t above z t for z < 0
+        U = static_cast<long long>(static_cast<unsigned long long>(static_cast<uint32_t>(z)) * tt -
+                                   (static_cast<unsigned long long>(z < 0 ? tt : 0u) << 32));
     const unsigned long long t = static_cast<unsigned long long>(sw.m) * static_cast<uint32_t>(U) + sw.h;
     const long long X = static_cast<long long>(sw.m) * static_cast<int>(U >> 32) + static_cast<uint32_t>(t >> 32);
-    if (FAST) return static_cast<int>(__funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s - 1));
-    // the quotient by 2^31 of the whole needs bit 31 of t too where s_sw = 0
-    const long long Y = sw.s > 0 ? X >> (sw.s - 1) : 2 * X + static_cast<long long>((t >> 31) & 1u);
-    return static_cast<int>(max(min(Y, 127ll), -127ll));
+    return static_cast<int>(__funnelshift_r(static_cast<uint32_t>(X), static_cast<uint32_t>(X >> 32), sw.s - 1));
 }
 
 // Byte transpose of a 4x4 block: y_c = [x0.b_c, x1.b_c, x2.b_c, x3.b_c].
@@ -217,7 +252,7 @@ __device__ __forceinline__ void dw_transpose4(uint32_t x0, uint32_t x1, uint32_t
 // shifted by i bytes.  A step makes one block of four outputs; the frame words
 // of the next step's new block are loaded before this step's arithmetic, so
 // their latency hides behind it.
-template <int K, bool FAST>
+template <int K, int FORM>
 __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *xb, uint32_t *yb,
                                             int cw, int ts, int te, const uint32_t (&wq)[4][(K + 3) / 4],
                                             const int (&mq)[4], const int (&sq)[4],
@@ -257,7 +292,7 @@ __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *x
                     const uint32_t win = i == 0 ? A[q][j] : __funnelshift_r(A[q][j], A[q + 1][j], 8 * i);
                     acc = __dp4a(static_cast<int>(win), static_cast<int>(wq[j][q]), acc);
                 }
-                o[i][j] = dw_out<FAST>(acc, mq[j], sq[j], hq[j], sw);
+                o[i][j] = dw_out<FORM>(acc, mq[j], sq[j], hq[j], sw);
             }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -275,8 +310,8 @@ __device__ __forceinline__ void dw4_segment(const DwParams &p, const uint32_t *x
 // channels); CTA: a contiguous run of frames_per_cta of the B T frames,
 // split at utterance boundaries (the zero padding of each utterance).  The
 // grid holds one CTA per resident slot, so there is no partial second wave.
-template <int K>
-__global__ void __launch_bounds__(DW4_THREADS, 10) dwconv_swish_x4_kernel(const DwParams p) {
+template <int K, int FORM, int CTAS>
+__global__ void __launch_bounds__(DW4_THREADS, CTAS) dwconv_swish_x4_kernel(const DwParams p) {
     pdl_launch_dependents();
     pdl_wait();   // the grid before this one on the stream: complete, memory visible
     constexpr int Q = (K + 3) / 4;
@@ -309,7 +344,7 @@ __global__ void __launch_bounds__(DW4_THREADS, 10) dwconv_swish_x4_kernel(const 
     }
     int mq[4], sq[4], bq[4];
     long long hq[4];
-    bool fast = p.sw_fast != 0;
+    bool fast = FORM == DW_FAST;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int c = 4 * c4 + j;
@@ -342,10 +377,12 @@ __global__ void __launch_bounds__(DW4_THREADS, 10) dwconv_swish_x4_kernel(const 
         const size_t base = static_cast<size_t>(b) * p.T * cw + c4;
         const uint32_t *xb = reinterpret_cast<const uint32_t *>(p.x) + base;
         uint32_t *yb = reinterpret_cast<uint32_t *>(p.y) + base;
-        if (fast)
-            dw4_segment<K, true>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
+        if (FORM == DW_FULL)
+            dw4_segment<K, DW_FULL>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
+        else if (fast)
+            dw4_segment<K, DW_FAST>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
         else
-            dw4_segment<K, false>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
+            dw4_segment<K, DW_WIDE>(p, xb, yb, cw, ts, te, wq, mq, sq, bq, hq, sw);
         f += static_cast<uint32_t>(te - ts);
     }
 }
