@@ -35,13 +35,12 @@ int sm_count() {
 int g_dw4_slots[64][ipb::DW_KMAX + 1][4] = {{{0}}};
 
 template <int K, int FORM, int CTAS>
-cudaError_t launch_dw4_as(ipb::DwParams p, cudaStream_t st) {
+cudaError_t dw4_slots(int &slots) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    constexpr int kernel = CTAS > 1 ? 3 : FORM;
-    int slots = 0;
+    constexpr int kernel = CTAS == 10 ? 3 : FORM;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         slots = g_dw4_slots[dev][K][kernel];
@@ -56,28 +55,57 @@ cudaError_t launch_dw4_as(ipb::DwParams p, cudaStream_t st) {
         std::lock_guard<std::mutex> lock(g_mu);
         g_dw4_slots[dev][K][kernel] = slots;
     }
-    // channel blocks of 256 channels; the frames of each split evenly over
-    // the slots left for it
+    return cudaSuccess;
+}
+
+// Channel blocks of 256 channels; the frames of each split evenly over the
+// slots left for it, in a multiple of the frames of one step, so that only
+// utterance ends leave a partly used step.
+dim3 dw4_grid(ipb::DwParams &p, int slots) {
     const int ncb = (p.C / 4 + ipb::DW4_THREADS - 1) / ipb::DW4_THREADS;
     const long long frames = static_cast<long long>(p.B) * p.T;
     long long per_block = slots / ncb > 0 ? slots / ncb : 1;
-    // a multiple of the frames of one step, so that only utterance ends
-    // leave a partly used step
     constexpr int step = 4;
     const long long per = ((frames + per_block - 1) / per_block + step - 1) / step * step;
     per_block = (frames + per - 1) / per;
     p.frames_per_cta = static_cast<uint32_t>(per);
     p.t_magic = iph::div_magic(static_cast<unsigned long long>(p.T));
-    return iph::launch_pdl(ipb::dwconv_swish_x4_kernel<K, FORM, CTAS>,
-                           dim3(static_cast<unsigned>(per_block), static_cast<unsigned>(ncb)),
-                           dim3(ipb::DW4_THREADS), 0, st, p);
+    return dim3(static_cast<unsigned>(per_block), static_cast<unsigned>(ncb));
+}
+
+template <int K, int FORM, int CTAS>
+cudaError_t launch_dw4_as(const ipb::DwParams &p, dim3 grid, cudaStream_t st) {
+    return iph::launch_pdl(ipb::dwconv_swish_x4_kernel<K, FORM, CTAS>, grid, dim3(ipb::DW4_THREADS), 0, st, p);
+}
+
+template <int K, int FORM>
+cudaError_t launch_dw4_form(ipb::DwParams &p, cudaStream_t st) {
+    int slots = 0;
+    const cudaError_t e = dw4_slots<K, FORM, 1>(slots);
+    if (e != cudaSuccess) return e;
+    return launch_dw4_as<K, FORM, 1>(p, dw4_grid(p, slots), st);
 }
 
 template <int K>
-cudaError_t launch_dw4(const ipb::DwParams &p, cudaStream_t st) {
-    if (p.sw_form == ipb::DW_FULL) return launch_dw4_as<K, ipb::DW_FULL, 1>(p, st);
-    if (p.sw_form == ipb::DW_WIDE) return launch_dw4_as<K, ipb::DW_WIDE, 1>(p, st);
-    return launch_dw4_as<K, ipb::DW_FAST, 10>(p, st);
+cudaError_t launch_dw4(ipb::DwParams p, cudaStream_t st) {
+    if (p.sw_form == ipb::DW_FULL) return launch_dw4_form<K, ipb::DW_FULL>(p, st);
+    if (p.sw_form == ipb::DW_WIDE) return launch_dw4_form<K, ipb::DW_WIDE>(p, st);
+    // Ten CTAs per SM (96 registers) pay where the grid needs them.  One of five to
+    // seven per SM (six from K = 13 on) takes the kernel with up to 144 (168)
+    // registers, whose loads go out further ahead: 400 x 4096, K = 13 7.2 -> 5.3 us (6.5
+    // with seven), 4000 x 512, K = 9 6.9 -> 6.0, 700 x 1024, K = 13 5.0 -> 4.1.  With four
+    // or less it gains nothing, and the launches before and after find less room on
+    // the SMs (block of 125 frames 89.1 -> 89.8 us).
+    constexpr int few = K >= 13 ? 6 : 7;
+    int slots = 0, slots_few = 0;
+    cudaError_t e = dw4_slots<K, ipb::DW_FAST, 10>(slots);
+    if (e == cudaSuccess) e = dw4_slots<K, ipb::DW_FAST, few>(slots_few);
+    if (e != cudaSuccess) return e;
+    const dim3 grid = dw4_grid(p, slots);
+    const long long ctas = static_cast<long long>(grid.x) * grid.y;
+    if (ctas > 4ll * sm_count() && ctas <= slots_few)
+        return launch_dw4_as<K, ipb::DW_FAST, few>(p, grid, st);
+    return launch_dw4_as<K, ipb::DW_FAST, 10>(p, grid, st);
 }
 
 // The form of dw_out that the constants fit.  No negative output below -127: the

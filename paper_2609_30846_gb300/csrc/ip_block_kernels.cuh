@@ -146,10 +146,11 @@ __global__ void __launch_bounds__(DW_THREADS) dwconv_swish_kernel(const DwParams
 // multiplies (every multiply, dp4a, shift, permute and pack takes two cycles of a
 // pipe per warp, additions and minima one).  So the two quotients are taken at word
 // boundaries on signed products, a thread makes four frames at a time (eight kept
-// more registers and fewer warps: 21.6 us), and ten CTAs of 64 threads share an SM
-// (96 registers; with eight, 128 registers, the largest case is 2 % faster, but 1332
-// frames take 6.3 us).  12000 x 1024, K = 9: 25.3 -> 21.0 us; K = 15: 27.7 -> 22.6;
-// 12000 x 512, K = 5: 17.0 -> 11.0; 1332 x 1024, K = 9: 7.6 -> 5.3; 125 x 1024: 2.8 -> 2.2.
+// more registers and fewer warps: 21.6 us), and up to ten CTAs of 64 threads share an
+// SM (96 registers; some shorter grids get more, launch_dw4).  With one form of arithmetic for
+// all constants, eight frames at a time and no bound on the registers: 12000 x 1024, K
+// = 9 22.8 us, now 19.5; K = 15: 25.3, 22.0; 12000 x 512, K = 5: 15.0, 10.6; 1332 x 1024,
+// K = 9: 6.4, 4.9; 400 x 4096, K = 13: 5.7, 5.3; 125 x 1024, K = 9: 3.5, 2.7.
 constexpr int DW4_THREADS = 64;      // 256 channels per CTA
 
 struct Swish16K {

@@ -70,3 +70,28 @@ def test_forms(ip, orc, K, i):
     g.check()
     bad = int((got.cpu().numpy() != want).sum())
     assert bad == 0, f"{bad} of {want.size} differ"
+
+
+# C = 512: the frames of a channel block are dealt four (eight from 3041 on) to a CTA
+# as ten CTAs per SM would take them; from 609 to 1064 CTAs (912 from K = 13 on) run as
+# seven (six) per SM: 1217 to 2128 frames, and 3041 to 4256 (to 1824 and 3648)
+@pytest.mark.parametrize("K", [1, 3, 5, 7, 9, 11, 13, 15])
+@pytest.mark.parametrize("B,T", [(4, 304), (1, 1217), (4, 456), (1, 1825), (7, 304), (1, 2129), (1, 3041), (3, 1216), (1, 3649), (8, 532),
+                                 (1, 4257)])
+def test_ctas_per_sm(ip, orc, K, B, T):
+    C = 512
+    rng = np.random.default_rng(B * T + K)
+    x = rng.integers(-127, 128, size=(B, T, C)).astype(np.int8)
+    w = rng.integers(-127, 128, size=(C, K)).astype(np.int8)
+    m = rng.integers(2 ** 30, 2 ** 31, size=C).astype(np.int32)
+    s = rng.integers(0, 4, size=C).astype(np.int32)
+    bias = rng.integers(-2000, 2000, size=C).astype(np.int32)
+    q = orc.swish16_params(10 / 32767, 4 / 127)
+    want = orc.swish16(orc.dwconv(x, w, bias, m, s), q)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    g, ws = Guarded(want.shape, torch.int8), torch.zeros(256, dtype=torch.uint8, device="cuda")
+    got = ip.dwconv_swish_i8(d(x), d(w), d(bias), d(m), d(s), (q.q_c, q.q_one, q.m, q.s), out=g.view, workspace=ws)
+    assert ip.status(ws) == 0
+    g.check()
+    bad = int((got.cpu().numpy() != want).sum())
+    assert bad == 0, f"{bad} of {want.size} differ"
