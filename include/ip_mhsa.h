@@ -79,7 +79,8 @@ typedef struct {
  * the calls that use it.  The caller zero-fills the workspace once before
  * its first use; ip_relpos_mhsa_status reads and clears it.  The workspace
  * also holds the work-item counters of the attention kernel (its CTAs claim
- * query tiles from them), which every call returns to zero when it ends;
+ * query tiles from them), which every call returns to zero when it ends, and
+ * one bit per SM, which calls leave in any state and any call can start from;
  * calls that share a workspace must not overlap on the GPU.
  * For T > 384 the size also counts a region for the int8 scores of every
  * resident CTA of the current device (4 warps x 16 rows x T, rounded up to
@@ -429,8 +430,10 @@ int ip_debug_set_stall_injection(int on);
  * quarter full, its tiles are done as four quarters of 16 rows, when at most
  * half full as two halves of 32 rows, whose warps split the keys of every
  * chunk and combine their row maxima, exponential sums and attn.V partial
- * sums.  0: no tile is split.  1: every tile in halves.  2 (or more): every
- * tile in quarters.  The outputs are the same bit for bit in every mode. */
+ * sums; and with two CTAs per SM, up to three quarters full, as one whole tile
+ * per SM and the others in quarters or halves beside them.  0: no tile is
+ * split.  1: every tile in halves.  2 (or more): every tile in quarters.  The
+ * outputs are the same bit for bit in every mode. */
 int ip_debug_set_split_mode(int mode);
 
 /* Test hook: nonzero makes the attention kernel take its general softmax

@@ -15,7 +15,6 @@
 
 namespace {
 
-constexpr size_t WS_HEADER = 256;          // error word and padding
 constexpr long long DEFAULT_TIMEOUT = 4000000000ll;   // ~2 s at 2 GHz
 long long g_timeout_cycles = DEFAULT_TIMEOUT;
 int g_stall_injection = 0;
@@ -31,9 +30,9 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 // The workspace holds the device error word of the calls that use it (byte
-// 0) and the attention kernel's item counters (bytes 64 and 128), which the
-// last CTA of every launch returns to zero.
-size_t ws_bytes() { return WS_HEADER; }
+// 0) and the attention kernel's item counters and SM bits (ipk::SCHED_BYTE on):
+// the last CTA of every launch returns the counters to zero, the bits stay.
+size_t ws_bytes() { return ipk::WS_HEADER; }
 
 int check_shape(int B, int H, int T, int dh) {
     if (dh != IP_DH) return IP_ERR_UNSUPPORTED;
@@ -302,7 +301,7 @@ int ip_relpos_mhsa_i8_ex(const int8_t *q, const int8_t *k, const int8_t *v, cons
     prm.out = out;
     prm.lengths = lengths;
     prm.err = err;
-    prm.sched = reinterpret_cast<unsigned int *>(static_cast<char *>(workspace) + 64);
+    prm.sched = reinterpret_cast<unsigned int *>(static_cast<char *>(workspace) + ipk::SCHED_BYTE);
     prm.B = B;
     prm.H = H;
     prm.T = T;

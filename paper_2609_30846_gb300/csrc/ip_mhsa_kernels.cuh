@@ -105,10 +105,7 @@ struct FusedParams {
     // the 2^split_log2 parts (32-row halves or 16-row quarters) of the tiles
     // from nwhole on.  With live_plan (a key-padding mask) the items are those
     // of LivePlan instead.
-    // Workspace words: [4 i] next item of list i (see claim), [16] CTAs done
-    // claiming, [32 ..] one bit per SM, flipped by each CTA that asks for its
-    // place on the SM.
-    unsigned int *sched;
+    unsigned int *sched;               // the workspace from byte SCHED_BYTE on
     int ntiles;                        // 64-row tiles per (b, h)
     unsigned long long tiles_magic;    // udiv_magic constant of ntiles
     unsigned long long heads_magic;    // udiv_magic constant of H
@@ -169,6 +166,23 @@ constexpr int ERR_TIMEOUT_EMPTY = 2;
 constexpr int ERR_TIMEOUT_READY = 4;
 constexpr int ERR_TIMEOUT_INJECTED = 8;
 constexpr long long DRAIN_CYCLES = 2000000000ll;
+
+// The first WS_HEADER bytes of the workspace: the error word (byte 0) and, from
+// SCHED_BYTE on, the 32-bit words of the item claims: the next item of list i at
+// SCHED_LIST i (see claim) and the CTAs done claiming at SCHED_DONE, which the last
+// CTA of a launch sets back to zero, and at SCHED_BITS one bit per SM, flipped by each
+// CTA that asks for its place on the SM and kept from launch to launch (any value is
+// valid).
+constexpr int WS_HEADER = 256;
+constexpr int SCHED_BYTE = 64;
+constexpr int SCHED_LIST = 4;
+constexpr int SCHED_LISTS = 3;
+constexpr int SCHED_DONE = 16;
+constexpr int SCHED_BITS = 32;
+constexpr int SCHED_BIT_WORDS = 8;      // a power of two; 256 SMs
+static_assert(SCHED_LIST * SCHED_LISTS <= SCHED_DONE && SCHED_DONE < SCHED_BITS &&
+                  SCHED_BYTE + 4 * (SCHED_BITS + SCHED_BIT_WORDS) <= WS_HEADER,
+              "the words end within the header");
 
 // ---------------------------------------------------------------- helpers --
 
@@ -1596,7 +1610,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
             } else {
                 if (mixed) end = phase == 0 ? nmain : (phase == 1 ? nwhole : n);
                 uint32_t x = 0;
-                if (lane == 0) x = atomicAdd(prm.sched + 4 * phase, 1u);
+                if (lane == 0) x = atomicAdd(prm.sched + SCHED_LIST * phase, 1u);
                 item = __shfl_sync(0xffffffffu, x, 0) + (phase == 0 ? 0u : (phase == 1 ? nmain : nwhole));
             }
             if (item < end) {
@@ -1612,7 +1626,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
                     uint32_t sm;
                     asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
                     const uint32_t bit = 1u << (sm & 31u);
-                    x = (atomicXor(prm.sched + 32 + ((sm >> 5) & 7u), bit) & bit) != 0u;
+                    x = (atomicXor(prm.sched + SCHED_BITS + ((sm >> 5) & (SCHED_BIT_WORDS - 1u)), bit) & bit) != 0u;
                 }
                 phase += static_cast<int>(__shfl_sync(0xffffffffu, x, 0));
             }
@@ -1641,10 +1655,10 @@ __global__ void __launch_bounds__(NTHREADS, 2)
         }
     };
     auto done_claiming = [&]() {
-        if (lane == 0 && atomicAdd(prm.sched + 16, 1u) == gridDim.x - 1) {
+        if (lane == 0 && atomicAdd(prm.sched + SCHED_DONE, 1u) == gridDim.x - 1) {
 #pragma unroll
-            for (int i = 0; i < 3; ++i) atomicExch(prm.sched + 4 * i, 0u);
-            atomicExch(prm.sched + 16, 0u);
+            for (int i = 0; i < SCHED_LISTS; ++i) atomicExch(prm.sched + SCHED_LIST * i, 0u);
+            atomicExch(prm.sched + SCHED_DONE, 0u);
         }
     };
 
