@@ -186,20 +186,6 @@ static_assert(SCHED_LIST * SCHED_LISTS <= SCHED_DONE && SCHED_DONE < SCHED_BITS 
 
 // ---------------------------------------------------------------- helpers --
 
-// Byte transpose of a 4x4 block: y_c = [x0.b_c, x1.b_c, x2.b_c, x3.b_c].
-__device__ __forceinline__ void transpose4(uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
-                                           uint32_t &y0, uint32_t &y1, uint32_t &y2,
-                                           uint32_t &y3) {
-    const uint32_t t0 = __byte_perm(x0, x1, 0x5140);
-    const uint32_t t1 = __byte_perm(x0, x1, 0x7362);
-    const uint32_t t2 = __byte_perm(x2, x3, 0x5140);
-    const uint32_t t3 = __byte_perm(x2, x3, 0x7362);
-    y0 = __byte_perm(t0, t2, 0x5410);
-    y1 = __byte_perm(t0, t2, 0x7632);
-    y2 = __byte_perm(t1, t3, 0x5410);
-    y3 = __byte_perm(t1, t3, 0x7632);
-}
-
 // Packs the low bytes of four values: [a.b0, b.b0, c.b0, d.b0].
 __device__ __forceinline__ uint32_t pack4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);

@@ -101,11 +101,6 @@ __device__ __forceinline__ uint32_t udiv_magic(uint32_t n, unsigned long long ma
     return magic == 0 ? n : static_cast<uint32_t>(__umul64hi(static_cast<unsigned long long>(n), magic));
 }
 
-// Barrier `id` (1..15) over the first `count` threads of the CTA.
-__device__ __forceinline__ void named_sync(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2,
                                         uint32_t &r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
